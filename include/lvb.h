@@ -374,8 +374,9 @@ int lvb_step_host(lvb_ctx *ctx, const float *pos_r, const float *vel, const floa
 /* Slots of lvb_trace. */
 #define LVB_TRACE_SLOTS 16
 /* Phases of the step kernel: 0 check (with the flagged particles'
- * updates), 1 rebuild passes, 2 re-layout, 3 tail (the DEM driver's
- * forces); separate kernels: 4 DEM integrate, 5 DEM forces, 6 full-build
+ * updates; inside dem_advance also the forces of the step before and the
+ * position half-step), 1 rebuild passes, 2 re-layout, 3 tail (the forces of
+ * the last step of a dem_advance launch); separate kernels: 4 DEM integrate, 5 DEM forces, 6 full-build
  * rows (init, store growth); inside the partial rebuild: 7 from the first
  * work item's start to the last one's end (patches and moves), 8 the
  * longest single work item. */
@@ -385,8 +386,7 @@ int lvb_step_host(lvb_ctx *ctx, const float *pos_r, const float *vel, const floa
  * each.  Synchronises. */
 int lvb_trace(lvb_ctx *ctx, uint64_t *sum_ns, uint64_t *count);
 
-/* lvb_set_option -- set an LVB_OPT_* value (synchronises if a cached graph
- * has to be rebuilt).  Errors: EINVAL. */
+/* lvb_set_option -- set an LVB_OPT_* value.  Errors: EINVAL. */
 int lvb_set_option(lvb_ctx *ctx, int32_t option, int64_t value);
 
 /* lvb_sync -- wait for the context's stream and return the sticky device

@@ -4,7 +4,7 @@ chunk, or one per block tile), and how the broad phase's check reads its
 inputs (register loads or a ring of bulk copies).
 
 Each candidate is a fresh context on the same batch from the same initial
-state; it runs ``warm`` steps (graph replays of DEM_GRAPH_STEPS steps), then
+state; it runs ``warm`` steps (launches of up to DEM_GRAPH_STEPS steps), then
 ``steps`` steps phase by phase, the broad phase of each between CUDA events
 on the context's stream: the tuner minimises the broad phase's time.  The
 search is coordinate-wise: the cell factor first (it changes the grid, so a
@@ -43,7 +43,7 @@ class Choice:
 
 def _trial(torch, lvb, scene_list, choice, warm, steps):
     """Broad-phase time per step of one candidate: `warm` steps of the DEM
-    driver (graphs), then `steps` steps phase by phase with CUDA events
+    driver, then `steps` steps phase by phase with CUDA events
     around each broad-phase launch (the quantity the candidates differ in:
     the cell factor changes the grid and the skins' cap, the other choices
     the broad phase's launch)."""

@@ -23,6 +23,40 @@ constexpr int kNumSMs = 152;
 constexpr int kThreads = 256;
 
 // ---------------------------------------------------------------------------
+// One step of the broad phase alone.  pos / vel / acc: the caller's
+// positions, velocities (policy input) and accelerations.  Launched
+// cooperatively with every block resident.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(kStepMaxThreads, 1)
+k_step(const float4 *__restrict__ pos, const float4 *vel, const float4 *acc,
+       const __grid_constant__ DevState sp)
+{
+    // the context's state read in place from the parameter space (uniform
+    // reads through the constant cache; no copy at the start)
+    const DevState &s = sp;
+    DevCounters *c = s.cnt;
+    const unsigned long long t0 = (s.trace && step_lead()) ? global_ns() : 0ULL;
+    // every thread reads the counters it needs (one broadcast load each, no
+    // block barrier before the check's loads); they are stable while the
+    // check runs
+    const unsigned err = c->err;
+    if (err & DERR_SYNC) return;   // a barrier failed earlier: the context is unusable
+    const bool inc = s.trigger == LVB_TRIGGER_PARTIAL && !(err & DERR_STORE);
+    const int step = (int)c->steps + 1, slot = step_slot(step);
+    __shared__ __align__(16) lvb_mlp_weights w_sh;
+    const bool net = s.skin_kind == LVB_SKIN_LEARNED;
+    if (net) weights_copy_async(&w_sh, s.mlp);
+    step_kernel_begin();
+    grid_barrier_begin(slot);
+    if (step_lead()) atomicAdd(&c->kernels, 1ULL);
+    if (s.check_regs) check_pass_regs(s, pos, vel, acc, inc, step, &c->nF_acc[slot]);
+    else check_pass_stream(s, pos, vel, acc, inc, step, &c->nF_acc[slot]);
+    if (net) weights_copy_wait();
+    if (!finish_step(s, &w_sh, pos, vel, acc, inc, step, slot, t0)) return;
+    flush_work(s);
+}
+
+// ---------------------------------------------------------------------------
 // Full-build kernels (init and store growth).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(kThreads)
@@ -574,11 +608,11 @@ int size_step(lvb_ctx *c)
     // the attribute belongs to the kernel, for every context of the process:
     // always the largest any block size needs
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_step<false, NoTail>,
+        e = cudaFuncSetAttribute(k_step,
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  check_smem_bytes(kStepMaxThreads));
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<false, NoTail>,
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step,
                                                           c->block_threads, smem);
     if (e != cudaSuccess) return from_cuda(e);
     if (per_sm < 1) return LVB_EDEVICE;
@@ -915,11 +949,11 @@ static int init_impl(lvb_ctx **out, int nscenes, const int64_t *offsets, int64_t
     if (e == cudaSuccess) e = dalloc(&s.bits, c->nwords);
     if (e == cudaSuccess) e = dalloc(&s.fid, n);
     if (nscenes > 1) {
-        if (e == cudaSuccess) e = dalloc(&s.sc_cnt, 2LL * nscenes);
+        if (e == cudaSuccess) e = dalloc(&s.sc_cnt, 3LL * nscenes);
         if (e == cudaSuccess) e = dalloc(&s.sfid, n);
         if (e == cudaSuccess) e = dalloc(&s.sfref, n);
         if (e == cudaSuccess) e = dalloc(&s.fsc, n);
-        if (e == cudaSuccess) e = cudaMemsetAsync(s.sc_cnt, 0, sizeof(int) * 2 * nscenes, st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(s.sc_cnt, 0, sizeof(int) * 3 * nscenes, st);
     }
     if (e == cudaSuccess) e = dalloc(&s.row_off, n);
     if (e == cudaSuccess) e = dalloc(&s.row_len, n);
@@ -1095,11 +1129,10 @@ int lvb_step(lvb_ctx *c, const float *pos_r, const float *vel, const float *acc)
         if (rc) return rc;
     }
     const cudaError_t e =
-        launch_coop(k_step<false, NoTail>, dim3(c->step_blocks), dim3(c->block_threads),
+        launch_coop(k_step, dim3(c->step_blocks), dim3(c->block_threads),
                     c->s.check_regs ? (size_t)0 : (size_t)check_smem_bytes(c->block_threads),
                     c->stream,
-                    (const float4 *)pos_r, (const float4 *)vel, a4, c->s, IntegrateArgs{},
-                    NoTail{});
+                    (const float4 *)pos_r, (const float4 *)vel, a4, c->s);
     return from_cuda(e);
 }
 
@@ -1539,7 +1572,7 @@ DevState step_state(lvb_ctx *c)
 
 void step_shape(lvb_ctx *c, int *blocks, int *threads)
 {
-    *blocks = c->step_blocks;
+    if (blocks) *blocks = c->step_blocks;
     *threads = c->block_threads;
 }
 
@@ -1559,7 +1592,7 @@ int grow_stores_if_asked(lvb_ctx *c)
     return grow_if_asked(c);
 }
 
-int graph_version(lvb_ctx *c)
+int step_version(lvb_ctx *c)
 {
     return c->version;
 }

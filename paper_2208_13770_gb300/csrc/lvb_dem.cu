@@ -2,11 +2,10 @@
 //
 // Per step: position half-step (x', v*), the broad-phase step at x'
 // (displacement check and partial rebuild), forces (narrow phase on the
-// list rows, linear spring-dashpot, walls, a', v').  dem_advance runs each
-// step as one cooperative launch of the broad phase's step kernel with the
-// half-step fused into its check pass and the forces as its tail phase;
-// dem_phase runs the three parts as separate launches (k_integrate,
-// lvb_step, k_forces), with identical results.  Forces are accumulated per row of the
+// list rows, linear spring-dashpot, walls, a', v').  dem_advance runs up to
+// DEM_GRAPH_STEPS steps as one cooperative launch (k_advance); dem_phase runs
+// the three parts as separate launches (k_integrate, lvb_step, k_forces), with
+// identical results.  Forces are accumulated per row of the
 // symmetric list, so each pair is evaluated once from each side and no
 // atomics are needed; both evaluations give exactly opposite forces.
 //
@@ -45,6 +44,13 @@ struct DemDev {
     float4 *omega, *alpha, *wstar;     // null without friction
     RowsView rows;
     int trace;                         // per-kernel trace (copied at launch)
+};
+
+// The two buffers of x, v, a (and, with friction, w, al) of k_advance, whose
+// steps read their partners' state in one and write their own in the
+// other; the first of each is the driver's own array.
+struct DemBuffers {
+    float4 *x[2], *v[2], *a[2], *w[2], *al[2];
 };
 
 __device__ __forceinline__ void dtr_enter(const DemDev &d, int slot)
@@ -97,71 +103,91 @@ __device__ __forceinline__ float lsd(const DemDev &d, float dl, float vn, float 
     return f;
 }
 
-__host__ __device__ __forceinline__ IntegrateArgs integrate_args(const DemDev &d)
-{
-    IntegrateArgs a;
-    a.pos = d.pos;
-    a.vel = d.vel;
-    a.acc = d.acc;
-    a.vstar = d.vstar;
-    a.omega = d.omega;
-    a.alpha = d.alpha;
-    a.wstar = d.wstar;
-    a.dt = d.dt;
-    a.half_dt2 = d.half_dt2;
-    a.specular = d.wall_kind == DEM_WALL_SPECULAR;
-    a.active = 1;
-    return a;
-}
-
+// The old state is read with streaming loads (evict first), so that the L2
+// keeps the new positions this kernel writes for the broad phase that
+// follows.
 __global__ void __launch_bounds__(kThreads)
 k_integrate(DemDev d)
 {
     const int i = blockIdx.x * kThreads + threadIdx.x;
     if (i == 0) atomicAdd(d.rows.kernels, 1ULL);
     dtr_enter(d, TR_INTEGRATE);
-    // the scene's geometry only for the specular walls (no load otherwise)
-    if (i < d.n)
-        integrate_one<true>(integrate_args(d),
-                      d.rows.sg[d.rows.nscenes == 1 || d.wall_kind != DEM_WALL_SPECULAR
-                                    ? 0
-                                    : d.rows.scene_of[i]],
-                      i);
+    if (i < d.n) {
+        float4 x = __ldcs(d.pos + i), v = __ldcs(d.vel + i), vs;
+        half_step(x, v, __ldcs(d.acc + i), vs, d.dt, d.half_dt2);
+        if (d.wall_kind == DEM_WALL_SPECULAR) {   // the scene's geometry only here
+            reflect(x, v, vs, d.rows.sg[d.rows.nscenes == 1 ? 0 : d.rows.scene_of[i]]);
+            d.vel[i] = v;
+        }
+        d.pos[i] = x;
+        d.vstar[i] = vs;
+        if (d.omega) d.wstar[i] = star_of(d.omega[i], d.alpha[i], d.dt);   // w*.w keeps 1/I
+    }
     dtr_exit(d, TR_INTEGRATE);
 }
 
 // Wall planes normal to one axis: x in [lo, hi], velocity component v.
 __device__ __forceinline__ float plane_force(const DemDev &d, float x, float v, float r, float lo,
-                                             float hi, float m)
+                                             float hi, float im)
 {
+    // a gap more than 1e-4 wider than the radius is none (the compensated
+    // difference is within 2^-24 of the plain one), and most particles
+    // have six of these
+    const float far = r * 1.0001f;
     float F = 0.0f, hh, ll;
-    two_diff(x, lo, hh, ll);                       // x - lo
-    const float dlo = __fsub_rn(r, hh) - ll;
-    if (dlo > 0.0f) F += lsd(d, dlo, v, m);
-    two_diff(hi, x, hh, ll);                       // hi - x
-    const float dhi = __fsub_rn(r, hh) - ll;
-    if (dhi > 0.0f) F -= lsd(d, dhi, -v, m);
+    if (!(__fsub_rn(x, lo) > far)) {
+        two_diff(x, lo, hh, ll);                       // x - lo
+        const float dlo = __fsub_rn(r, hh) - ll;
+        if (dlo > 0.0f) F += lsd(d, dlo, v, 1.0f / im);
+    }
+    if (!(__fsub_rn(hi, x) > far)) {
+        two_diff(hi, x, hh, ll);                       // hi - x
+        const float dhi = __fsub_rn(r, hh) - ll;
+        if (dhi > 0.0f) F -= lsd(d, dhi, -v, 1.0f / im);
+    }
     return F;
 }
 
-// One contact of the narrow phase (Eq. delta) and its force: particle i at
-// xi with v* and 1/m in vi, against partner j of its row.  Returns false
-// when the two do not overlap (delta <= 0); else the overlap dl (compensated
-// binary32), the unit normal n (from j to i) and the normal force f on i
-// along n (linear spring-dashpot, damping on the normal component of
-// v*_i - v*_j).
-__device__ __forceinline__ bool contact_pair(const DemDev &d, float4 xi, float4 vi, int j,
-                                             float &dl, float n[3], float &f)
+// v* (or w*) of a partner: as the half-step stored it, or worked out again
+// from the state before the half-step, which a kernel that has already
+// written newer v and a elsewhere still holds (the same roundings).
+struct StoredStar {
+    const float4 *vs;
+    __device__ __forceinline__ float4 operator()(int j) const { return vs[j]; }
+};
+
+struct DerivedStar {
+    const float4 *v, *a;
+    float dt;
+    __device__ __forceinline__ float4 operator()(int j) const { return star_of(v[j], a[j], dt); }
+};
+
+// Whether two particles may overlap: the plain distance against the radii
+// with a margin far above its rounding.
+__device__ __forceinline__ bool may_touch(float4 xi, float4 xj)
 {
-    const float4 xj = d.pos[j];
+    const float hx = __fsub_rn(xi.x, xj.x), hy = __fsub_rn(xi.y, xj.y), hz = __fsub_rn(xi.z, xj.z);
+    const float Rr = xi.w + xj.w;
+    return !(hx * hx + hy * hy + hz * hz > Rr * Rr * 1.0001f);
+}
+
+// One contact of the narrow phase (Eq. delta) and its force: particle i at
+// xi with v* and 1/m in vi, against partner j of its row at xj.  Returns false
+// when the two do not overlap (delta <= 0); else the overlap dl (compensated
+// binary32), the unit normal n (from j to i), the normal force f on i
+// along n (linear spring-dashpot, damping on the normal component of
+// v*_i - v*_j), the partner's v* and the pair's effective mass.
+template <class Star>
+__device__ __forceinline__ bool contact_pair(const DemDev &d, const Star &star, float4 xi,
+                                             float4 vi, int j, float4 xj, float &dl, float n[3],
+                                             float &f, float4 &vj, float &meff)
+{
+    if (!may_touch(xi, xj)) return false;   // before the compensated distance
+    vj = star(j);   // loaded under the arithmetic: what may touch mostly does
     float h[3], l[3];
     two_diff(xi.x, xj.x, h[0], l[0]);
     two_diff(xi.y, xj.y, h[1], l[1]);
     two_diff(xi.z, xj.z, h[2], l[2]);
-    // cheap reject before the compensated distance
-    const float Rr = xi.w + xj.w;
-    const float d2 = h[0] * h[0] + h[1] * h[1] + h[2] * h[2];
-    if (d2 > Rr * Rr * 1.0001f) return false;
     float s0, corr;
     norm_dd(h, l, s0, corr);
     float Rh, Rl;
@@ -172,9 +198,8 @@ __device__ __forceinline__ bool contact_pair(const DemDev &d, float4 xi, float4 
     n[0] = (h[0] + l[0]) * inv;
     n[1] = (h[1] + l[1]) * inv;
     n[2] = (h[2] + l[2]) * inv;
-    const float4 vj = d.vstar[j];
     const float vn = (vi.x - vj.x) * n[0] + (vi.y - vj.y) * n[1] + (vi.z - vj.z) * n[2];
-    const float meff = 1.0f / (vi.w + vj.w);
+    meff = 1.0f / (vi.w + vj.w);
     f = lsd(d, dl, vn, meff);
     return true;
 }
@@ -190,11 +215,9 @@ __device__ __forceinline__ float dot_rn(float ax, float ay, float az, const floa
 // explicitly (no contraction), in an order that is exactly sign-symmetric
 // under exchanging i and j (n -> -n), so that j's record stays exactly -h.
 __device__ __forceinline__ float3 tangential(const DemDev &d, float ri, float4 vi, float4 wi,
-                                             int j, const float n[3], float fn, float meff,
-                                             float4 &h)
+                                             float rj, float4 vj, float4 wj, const float n[3],
+                                             float fn, float meff, float4 &h)
 {
-    const float4 vj = d.vstar[j], wj = d.wstar[j];
-    const float rj = d.pos[j].w;
     // s = r_i w_i + r_j w_j, c = s x n: the contact point's rotational velocity
     const float sx = __fadd_rn(__fmul_rn(ri, wi.x), __fmul_rn(rj, wj.x));
     const float sy = __fadd_rn(__fmul_rn(ri, wi.y), __fmul_rn(rj, wj.y));
@@ -234,149 +257,367 @@ __device__ __forceinline__ float3 tangential(const DemDev &d, float ri, float4 v
     return make_float3(Fx, Fy, Fz);
 }
 
-// Narrow phase on the row of particle i + walls + velocity finish; the
-// friction form (fric) also the tangential law, torques and rotation.
-// kEarly (the forces as a kernel of their own, 32 registers): the row
-// bounds and the scene of i are loaded with the particle's own state, not
-// after the error word and the row walk; the fused tail keeps the late
-// loads (fewer registers held across the walk).
-template <bool fric, bool kEarly = false>
-__device__ __forceinline__ void forces_body(const DemDev &d, int i)
+// Adds the contact of row entry e (partner j at xj) to the force on i in F and,
+// with friction, to the torque in T.
+template <bool kFric, class Star>
+__device__ __forceinline__ void add_contact(const DemDev &d, const Star &star, const Star &spin,
+                                            float4 xi, float4 vi, int i, int e, int j, float4 xj,
+                                            float F[3], float T[3])
 {
-    const float4 xi = d.pos[i];
-    const float4 vi = d.vstar[i];
-    const float4 a = d.acc[i];
-    float4 v = d.vel[i];
-    const float im_i = vi.w;
-    float Fx = 0.f, Fy = 0.f, Fz = 0.f;
-    float Tx = 0.f, Ty = 0.f, Tz = 0.f;
-    const float4 wi = fric ? d.wstar[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const bool walls = d.wall_kind == DEM_WALL_BOX || d.wall_kind == DEM_WALL_DRUM;
-    int sc_i = 0, off = 0, len = 0;
-    if (kEarly) {   // in range either way; used only as below
-        sc_i = walls && d.rows.nscenes > 1 ? d.rows.scene_of[i] : 0;
-        off = d.rows.row_off[i];
-        len = min(d.rows.row_len[i], d.rows.row_cap[i]);
+    float4 vj;
+    float dl, n[3], f, meff;
+    if (!contact_pair(d, star, xi, vi, j, xj, dl, n, f, vj, meff)) {
+        if (kFric) d.rows.hist[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+        return;
     }
-    // after a row store that failed even a tight re-layout (LVB_EOVERFLOW)
-    // the row offsets no longer fit the store: the rows are not read
-    if (d.contacts_on && !(d.rows.cnt->err & DERR_STORE)) {
-        if (!kEarly) {
-            off = d.rows.row_off[i];
-            len = min(d.rows.row_len[i], d.rows.row_cap[i]);
-        }
-        for (int e = 0; e < len; ++e) {
-            const int j = d.rows.col[off + e];
-            if (j < 0) continue;            // a removed pair's slot
-            float dl, n[3], f;
-            if (!contact_pair(d, xi, vi, j, dl, n, f)) {
-                if (fric) d.rows.hist[off + e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                continue;
-            }
-            Fx += f * n[0];
-            Fy += f * n[1];
-            Fz += f * n[2];
-            if (fric) {
-                float4 h = d.rows.hist[off + e];
-                const float meff = 1.0f / (im_i + d.vstar[j].w);
-                const float3 Ft = tangential(d, xi.w, vi, wi, j, n, f, meff, h);
-                d.rows.hist[off + e] = h;
-                Fx += Ft.x;
-                Fy += Ft.y;
-                Fz += Ft.z;
-                // torque -r_i n x F_t
-                Tx -= xi.w * (n[1] * Ft.z - n[2] * Ft.y);
-                Ty -= xi.w * (n[2] * Ft.x - n[0] * Ft.z);
-                Tz -= xi.w * (n[0] * Ft.y - n[1] * Ft.x);
-            }
-        }
+    F[0] += f * n[0];
+    F[1] += f * n[1];
+    F[2] += f * n[2];
+    if (kFric) {
+        float4 h = d.rows.hist[e];
+        const float3 Ft = tangential(d, xi.w, vi, spin(i), xj.w, vj, spin(j), n, f, meff, h);
+        d.rows.hist[e] = h;
+        F[0] += Ft.x;
+        F[1] += Ft.y;
+        F[2] += Ft.z;
+        // torque -r_i n x F_t
+        T[0] -= xi.w * (n[1] * Ft.z - n[2] * Ft.y);
+        T[1] -= xi.w * (n[2] * Ft.x - n[0] * Ft.z);
+        T[2] -= xi.w * (n[0] * Ft.y - n[1] * Ft.x);
     }
-    const float r = xi.w;
-    if (walls) {
-        if (!kEarly && d.rows.nscenes > 1) sc_i = d.rows.scene_of[i];
-        const SceneGeom &g = d.rows.sg[sc_i];
-        const float m = 1.0f / im_i;
-        if (d.wall_kind == DEM_WALL_BOX) {
-            Fx += plane_force(d, xi.x, vi.x, r, g.lo[0], g.hi[0], m);
-            Fz += plane_force(d, xi.z, vi.z, r, g.lo[2], g.hi[2], m);
+}
+
+// The contacts of row i (off, len; its partners at X) in row order.  The row
+// is read four entries at a time (rows start on 16 bytes) and the four
+// partners' positions together, so that a row of up to four costs two memory
+// latencies; only the few that may touch are taken up again, one after
+// another (their positions then come from the L1).
+template <bool kFric, class Star>
+__device__ __forceinline__ void row_forces(const DemDev &d, const float4 *X, const Star &star,
+                                           const Star &spin, float4 xi, float4 vi, int i, int off,
+                                           int len, float F[3], float T[3])
+{
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int e0 = 0; e0 < len; e0 += 4) {
+        const int4 j4 = *reinterpret_cast<const int4 *>(d.rows.col + off + e0);
+        float4 xj[4];
+        xj[0] = j4.x >= 0 ? X[j4.x] : zero;
+        xj[1] = j4.y >= 0 ? X[j4.y] : zero;
+        xj[2] = j4.z >= 0 ? X[j4.z] : zero;
+        xj[3] = j4.w >= 0 ? X[j4.w] : zero;
+        unsigned m = 0;
+        if (j4.x >= 0 && may_touch(xi, xj[0])) m |= 1u;
+        if (j4.y >= 0 && may_touch(xi, xj[1])) m |= 2u;
+        if (j4.z >= 0 && may_touch(xi, xj[2])) m |= 4u;
+        if (j4.w >= 0 && may_touch(xi, xj[3])) m |= 8u;
+        if (kFric) {   // entries out of contact keep no spring
+            const int e = off + e0;
+            if (j4.x >= 0 && !(m & 1u)) d.rows.hist[e] = zero;
+            if (j4.y >= 0 && !(m & 2u)) d.rows.hist[e + 1] = zero;
+            if (j4.z >= 0 && !(m & 4u)) d.rows.hist[e + 2] = zero;
+            if (j4.w >= 0 && !(m & 8u)) d.rows.hist[e + 3] = zero;
         }
-        Fy += plane_force(d, xi.y, vi.y, r, g.lo[1], g.hi[1], m);   // box side / drum caps
-        if (d.wall_kind == DEM_WALL_DRUM) {
-            float h[3], l[3];
-            two_diff(xi.x, d.drum_cx, h[0], l[0]);
-            h[1] = 0.0f;
-            l[1] = 0.0f;
-            two_diff(xi.z, d.drum_cz, h[2], l[2]);
-            float s0, corr;
-            norm_dd(h, l, s0, corr);
-            // delta = r + rho - R, rho = s0 + corr; (s0 - R) is exact near the wall
-            const float t = __fsub_rn(s0, d.drum_R);
-            const float dl = __fadd_rn(t, r) + corr;
-            if (dl > 0.0f && s0 > 0.0f) {
-                const float inv = 1.0f / s0;
-                const float nx = -(h[0] + l[0]) * inv, nz = -(h[2] + l[2]) * inv;
-                const float vn = vi.x * nx + vi.z * nz;
-                const float f = lsd(d, dl, vn, m);
-                Fx += f * nx;
-                Fz += f * nz;
-            }
+        while (m) {
+            const int u = __ffs(m) - 1;
+            m &= m - 1;
+            const int j = u < 2 ? (u == 0 ? j4.x : j4.y) : (u == 2 ? j4.z : j4.w);
+            add_contact<kFric>(d, star, spin, xi, vi, i, off + e0 + u, j, X[j], F, T);
         }
     }
-    const float4 an = make_float4(Fx * im_i + d.g[0], Fy * im_i + d.g[1], Fz * im_i + d.g[2],
+}
+
+// The walls' forces on particle i, added to F; im: 1/m.
+__device__ __forceinline__ void wall_forces(const DemDev &d, float4 xi, float4 vi, int sc_i,
+                                            float F[3])
+{
+    if (d.wall_kind != DEM_WALL_BOX && d.wall_kind != DEM_WALL_DRUM) return;
+    const float r = xi.w, im = vi.w;
+    const SceneGeom &g = d.rows.sg[sc_i];
+    if (d.wall_kind == DEM_WALL_BOX) {
+        F[0] += plane_force(d, xi.x, vi.x, r, g.lo[0], g.hi[0], im);
+        F[2] += plane_force(d, xi.z, vi.z, r, g.lo[2], g.hi[2], im);
+    }
+    F[1] += plane_force(d, xi.y, vi.y, r, g.lo[1], g.hi[1], im);   // box side / drum caps
+    if (d.wall_kind == DEM_WALL_DRUM) {
+        // well inside the drum (by 1e-4 of its free radius, far above the
+        // rounding of the plain distance): no wall
+        const float px = __fsub_rn(xi.x, d.drum_cx), pz = __fsub_rn(xi.z, d.drum_cz);
+        const float in = (d.drum_R - r) * 0.9999f;
+        if (in > 0.0f && px * px + pz * pz < in * in) return;
+        float h[3], l[3];
+        two_diff(xi.x, d.drum_cx, h[0], l[0]);
+        h[1] = 0.0f;
+        l[1] = 0.0f;
+        two_diff(xi.z, d.drum_cz, h[2], l[2]);
+        float s0, corr;
+        norm_dd(h, l, s0, corr);
+        // delta = r + rho - R, rho = s0 + corr; (s0 - R) is exact near the wall
+        const float t = __fsub_rn(s0, d.drum_R);
+        const float dl = __fadd_rn(t, r) + corr;
+        if (dl > 0.0f && s0 > 0.0f) {
+            const float inv = 1.0f / s0;
+            const float nx = -(h[0] + l[0]) * inv, nz = -(h[2] + l[2]) * inv;
+            const float vn = vi.x * nx + vi.z * nz;
+            const float f = lsd(d, dl, vn, 1.0f / im);
+            F[0] += f * nx;
+            F[2] += f * nz;
+        }
+    }
+}
+
+// a' = F / m + g and v' = v + (a + a') dt / 2 (v.w, 1/m, kept)
+__device__ __forceinline__ float4 finish_velocity(const DemDev &d, const float F[3], float im,
+                                                  float4 a, float4 &v)
+{
+    const float4 an = make_float4(F[0] * im + d.g[0], F[1] * im + d.g[1], F[2] * im + d.g[2],
                                   0.0f);
     v.x += (a.x + an.x) * d.half_dt;
     v.y += (a.y + an.y) * d.half_dt;
     v.z += (a.z + an.z) * d.half_dt;
+    return an;
+}
+
+// al' = T / I, w' = w + (al + al') dt / 2 (w.w, 1/I, kept)
+__device__ __forceinline__ float4 finish_spin(const DemDev &d, const float T[3], float4 al,
+                                              float4 &w)
+{
+    const float4 aln = make_float4(T[0] * w.w, T[1] * w.w, T[2] * w.w, 0.0f);
+    w.x += (al.x + aln.x) * d.half_dt;
+    w.y += (al.y + aln.y) * d.half_dt;
+    w.z += (al.z + aln.z) * d.half_dt;
+    return aln;
+}
+
+// Whether the walls need the scene of each particle, and the scene of i if so.
+__device__ __forceinline__ bool wall_scenes(const DemDev &d)
+{
+    return d.wall_kind != DEM_WALL_NONE && d.rows.nscenes > 1;
+}
+
+__device__ __forceinline__ int wall_scene(const DemDev &d, int i)
+{
+    return wall_scenes(d) ? d.rows.scene_of[i] : 0;
+}
+
+// The forces phase of particle i from the stored x', v* (and w*); the state
+// before the step's forces is v, a (w, al), the new one goes to d.vel, d.acc
+// (d.omega, d.alpha).  rows: the rows may be read (contacts on, store not failed:
+// after LVB_EOVERFLOW the row offsets no longer fit the store).  The row
+// bounds and the scene are loaded with the particle's own state.
+template <bool kFric>
+__device__ __forceinline__ void forces_body(const DemDev &d, int i, const float4 *vin,
+                                            const float4 *ain, const float4 *win,
+                                            const float4 *alin)
+{
+    const float4 xi = d.pos[i];
+    const float4 vi = d.vstar[i];
+    const float4 a = ain[i];
+    float4 v = vin[i];
+    const int sc_i = wall_scene(d, i), off = d.rows.row_off[i];
+    int len = min(d.rows.row_len[i], d.rows.row_cap[i]);
+    if (!d.contacts_on || (d.rows.cnt->err & DERR_STORE)) len = 0;
+    const StoredStar star{d.vstar}, spin{d.wstar};
+    float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
+    row_forces<kFric>(d, d.pos, star, spin, xi, vi, i, off, len, F, T);
+    wall_forces(d, xi, vi, sc_i, F);
+    d.acc[i] = finish_velocity(d, F, vi.w, a, v);
     d.vel[i] = v;
-    d.acc[i] = an;
-    if (fric) {   // al' = T / I, w' = w + (al + al') dt / 2
-        float4 w = d.omega[i];
-        const float4 al = d.alpha[i];
-        const float4 aln = make_float4(Tx * w.w, Ty * w.w, Tz * w.w, 0.0f);
-        w.x += (al.x + aln.x) * d.half_dt;
-        w.y += (al.y + aln.y) * d.half_dt;
-        w.z += (al.z + aln.z) * d.half_dt;
+    if (kFric) {
+        float4 w = win[i];
+        d.alpha[i] = finish_spin(d, T, alin[i], w);
         d.omega[i] = w;
-        d.alpha[i] = aln;
     }
 }
 
-// The friction form is a separate function, so that its registers do not
-// weigh on the kernels that run without it.
-static __device__ __noinline__ void forces_one_fric(const DemDev &d, int i)
-{
-    forces_body<true>(d, i);
-}
-
-template <bool kEarly = false>
-__device__ __forceinline__ void forces_one(const DemDev &d, int i)
-{
-    if (d.omega) forces_one_fric(d, i);
-    else forces_body<false, kEarly>(d, i);
-}
-
-// Forces as a separate kernel, one thread per particle.  Eight blocks per
-// SM (32 registers, a few spilled): the row walks are dependent loads, and
-// full occupancy hides them better (-10% on the batched workload).
-__global__ void __launch_bounds__(kThreads, 8)
+// Forces as a separate kernel, one thread per particle.  Bound by the row
+// walks' dependent loads: a row taken four entries at a time wants 48 registers
+// (five blocks an SM; friction 64, four blocks), which beats the full
+// occupancy of an entry-by-entry walk in 32 (6.2M batch 168 -> 160 us, 2M drum
+// 82 -> 77 us, 1M drum with friction 199 -> 124 us).
+template <bool kFric>
+__global__ void __launch_bounds__(kThreads, kFric ? 4 : 5)
 k_forces(DemDev d)
 {
     const int i = blockIdx.x * kThreads + threadIdx.x;
     if (i == 0) atomicAdd(d.rows.kernels, 1ULL);
     dtr_enter(d, TR_FORCES);
-    if (i < d.n) forces_one<true>(d, i);
+    if (i < d.n) forces_body<kFric>(d, i, d.vel, d.acc, d.omega, d.alpha);
     dtr_exit(d, TR_FORCES);
 }
 
-// Forces as the tail phase of the fused step kernel (grid-stride).
-struct DemTail {
-    static constexpr bool kActive = true;
-    DemDev d;
-    __device__ void operator()(int t, int nt) const
-    {
-        for (int i = t; i < d.n; i += nt) forces_one(d, i);
+// One pass over the particles of k_advance.  kForces: the forces at (x, v*)
+// of the step before, with v* worked out again from v and a, its a' and v',
+// then the position half-step and the displacement check of this step;
+// else the half-step and the check only (the first step of a launch).
+// Reads the state in one of the two buffers of each array, bx for x, bv for
+// v, a (w, al), and writes x to buffer ox and the others to bv ^ 1: partners'
+// x, v, a are read all through the pass, so none of them may be written
+// there (the half-step alone touches no partner and runs in place).
+// Each warp takes chunks of 32 consecutive particles, warp w of block b the
+// chunks w * grid + b, + all warps, ... (so that a last, partial round
+// spreads over all SMs).  The chain of dependent loads is row bounds, row,
+// partners' positions, at 32 warps an SM (64 registers a thread): the bounds are
+// loaded a chunk ahead and the row's first sector is asked for from DRAM
+// then (512 scenes, 6.2M particles: 202 -> 185 -> 174 us a pass).  A ring of
+// asynchronous copies of x, v, a and the reference state in shared memory
+// was slower (the L1 that it displaces holds the rows and partners: 186 us
+// there, the 2M drum 82 -> 107 us), and so were L2 prefetches of them.
+template <bool kFric, bool kForces>
+__device__ __forceinline__ void advance_pass(const DevState &s, const DemDev &d,
+                                             const DemBuffers &b, int bx, int ox, int bv,
+                                             bool rows, bool keep_star, bool inc, int step,
+                                             int *nF_acc)
+{
+    __shared__ int pend_id[kStepMaxThreads / 32][kPending];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    Pending pd{pend_id[warp], 0};
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    const bool scenes = wall_scenes(d), walk = kForces && rows;
+    auto bounds = [&](int c, int &o, int &l) {
+        const int i = c * 32 + lane;
+        o = l = 0;
+        if (walk && i < s.n) {
+            o = s.row_off[i];
+            l = s.row_len[i];   // at most the capacity between steps: a row that
+                                // outgrew it was laid out anew
+        }
+    };
+    int c = warp * gridDim.x + blockIdx.x, off, len;
+    bounds(c, off, len);
+    for (; c < s.nwords; c += nw) {
+        int off1, len1;   // the next chunk's
+        bounds(c + nw, off1, len1);
+        const int cu[1] = {c * 32};
+        const int i = cu[0] + lane;
+        bool f[1] = {false};
+        if (i < s.n) {
+            float4 x = b.x[bx][i], v = b.v[bv][i], a = b.a[bv][i], w, al;
+            const float4 q = __ldcs(s.ref + i);   // read once: evicted first
+            const int sc = scenes ? d.rows.scene_of[i] : 0;
+            if (kForces) {
+                float F[3] = {0.f, 0.f, 0.f}, Tq[3] = {0.f, 0.f, 0.f};
+                const float4 vi = star_of(v, a, d.dt);
+                if (len > 0) {
+                    const DerivedStar star{b.v[bv], b.a[bv], d.dt},
+                        spin{b.w[bv], b.al[bv], d.dt};
+                    row_forces<kFric>(d, b.x[bx], star, spin, x, vi, i, off, len, F, Tq);
+                }
+                wall_forces(d, x, vi, sc, F);
+                a = finish_velocity(d, F, vi.w, a, v);
+                __stcs(&b.a[bv ^ 1][i], a);   // read again a whole pass later
+                if (kFric) {
+                    w = b.w[bv][i];
+                    al = finish_spin(d, Tq, b.al[bv][i], w);
+                    b.w[bv ^ 1][i] = w;
+                    b.al[bv ^ 1][i] = al;
+                }
+            } else {
+                if (kFric) {
+                    w = b.w[bv][i];
+                    al = b.al[bv][i];
+                }
+            }
+            float4 vs;
+            half_step(x, v, a, vs, d.dt, d.half_dt2);
+            const bool mirror = d.wall_kind == DEM_WALL_SPECULAR;
+            if (mirror) reflect(x, v, vs, s.sg[sc]);
+            b.x[ox][i] = x;
+            if (kForces) __stcs(&b.v[bv ^ 1][i], v);
+            else if (mirror) b.v[bv][i] = v;
+            f[0] = violates(x, q);
+            if (!(isfinite(x.x) && isfinite(x.y) && isfinite(x.z)))
+                atomicOr(&s.cnt->err, DERR_NAN);
+            // v* for whoever reads it: the updates of this step, or (the
+            // launch's last step) the forces and the caller
+            if (keep_star || f[0]) {
+                d.vstar[i] = vs;
+                if (kFric) d.wstar[i] = star_of(w, al, d.dt);
+            }
+        }
+        flag_chunks<1>(s, cu, f, b.x[ox], d.vstar, nullptr, inc, step, nF_acc, pd);
+        off = off1;
+        len = len1;
+        if (len > 0) asm volatile("prefetch.global.L2 [%0];" ::"l"(s.col + off));
     }
-};
+    flush_pending_final(s, pd, b.x[ox], d.vstar, nullptr, inc, step, nF_acc);
+}
+
+// The rest of a step as a call of its own: what it keeps in registers does
+// not displace the pass's.  To a call the kernel's parameter is memory like
+// any other, cached in an L1 that every grid barrier empties, so the phases
+// after the pass read the context's state from a copy in shared memory
+// (settling 200k 24.6 -> 23.0 us a step).
+static __shared__ DevState s_state;
+
+static __device__ __noinline__ bool rest_of_step(const lvb_mlp_weights *w_sh, const float4 *pos,
+                                                 const float4 *vel, const float4 *acc, bool inc,
+                                                 int step, int slot, unsigned long long t0)
+{
+    return finish_step(s_state, w_sh, pos, vel, acc, inc, step, slot, t0);
+}
+
+// `steps` whole DEM steps as one cooperative launch, all blocks resident.
+// What bounds a step here is the traffic of the state and, for small runs,
+// the launches and barriers; so one pass over the particles does the forces
+// of a step and the half-step and check of the next (x, v, a and the
+// reference state read once, x, v, a written once: 112 bytes a particle plus
+// its row, where three phases move 204), and only a grid barrier lies
+// between the steps (two when something was flagged).
+// The state goes back and forth between two buffers and ends in d.pos, d.vel,
+// d.acc: the half-step of the first step writes x to the buffer from which
+// the steps - 1 passes that follow end there, the last forces write d.vel and
+// d.acc.  Those read v* (and w*) as the last pass stored it, so they need no
+// second buffer.
+template <bool kFric>
+__global__ void __launch_bounds__(kStepMaxThreads, 1)
+k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
+          const __grid_constant__ DemBuffers b, int steps)
+{
+    DevCounters *c = s.cnt;
+    const unsigned err0 = c->err;
+    if (err0 & DERR_SYNC) return;   // a barrier failed earlier: the context is unusable
+    int step = (int)c->steps, bx = 0, bv = 0;   // the buffers that hold the state
+    __shared__ __align__(16) lvb_mlp_weights w_sh;
+    const bool net = s.skin_kind == LVB_SKIN_LEARNED;
+    if (net) weights_copy_async(&w_sh, s.mlp);
+    step_kernel_begin();
+    static_assert(sizeof(DevState) % 4 == 0, "copied in words");
+    for (int t = threadIdx.x; t < (int)(sizeof(DevState) / 4); t += blockDim.x)
+        reinterpret_cast<unsigned *>(&s_state)[t] = reinterpret_cast<const unsigned *>(&s)[t];
+    if (step_lead()) atomicAdd(&c->kernels, 1ULL);
+    // v* of everyone at every step where the trigger may update anyone
+    const bool star_always = s.trigger != LVB_TRIGGER_PARTIAL || s.early_beta < 1.0f;
+    for (int k = 1; k <= steps; ++k) {
+        const unsigned long long t0 = (s.trace && step_lead()) ? global_ns() : 0ULL;
+        const unsigned err = k == 1 ? err0 : *(volatile unsigned *)&c->err;
+        const bool store_ok = !(err & DERR_STORE);
+        const bool inc = s.trigger == LVB_TRIGGER_PARTIAL && store_ok;
+        const bool star = star_always || k == steps;
+        const int slot = step_slot(++step);
+        grid_barrier_begin(slot);
+        int *nF_acc = &c->nF_acc[slot];
+        if (k == 1) {
+            const int ox = ~steps & 1;
+            advance_pass<kFric, false>(s, d, b, 0, ox, 0, false, star, inc, step, nF_acc);
+            bx = ox;
+            if (net) weights_copy_wait();
+        } else {
+            advance_pass<kFric, true>(s, d, b, bx, bx ^ 1, bv, store_ok && d.contacts_on, star,
+                                      inc, step, nF_acc);
+            bx ^= 1;
+            bv ^= 1;
+        }
+        if (!rest_of_step(&w_sh, b.x[bx], d.vstar, b.a[bv], inc, step, slot, t0)) return;
+    }
+    flush_work(s);
+    const unsigned long long t3 = (s.trace && step_lead()) ? global_ns() : 0ULL;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.n; i += gridDim.x * blockDim.x)
+        forces_body<kFric>(d, i, b.v[bv], b.a[bv], b.w[bv], b.al[bv]);
+    if (s.trace) {
+        if (!grid_barrier(s)) return;
+        if (step_lead()) trace_add(c, TR_TAIL, t3, global_ns());
+    }
+}
 
 // The contacts of the current state, each pair once (i < j from row i),
 // with the force on i and the overlap; positions in the output from one
@@ -397,8 +638,10 @@ k_contact_list(DemDev d, unsigned long long *cnt, long long cap, int *ci, int *c
         const int j = d.rows.col[off + e];
         // a removed pair's slot, or (one side only) the pair from j's row
         if (j < 0 || (!both && j <= i)) continue;
-        float dl, n[3], f;
-        if (!contact_pair(d, xi, vi, j, dl, n, f)) continue;
+        float dl, n[3], f, meff;
+        float4 vj;
+        const float4 xj = d.pos[j];
+        if (!contact_pair(d, StoredStar{d.vstar}, xi, vi, j, xj, dl, n, f, vj, meff)) continue;
         float Ft[3] = {0.f, 0.f, 0.f}, h[3] = {0.f, 0.f, 0.f};
         if (fric) {
             // F_t = -k_t xi - gamma_t v_t from the spring as the step left it
@@ -406,8 +649,8 @@ k_contact_list(DemDev d, unsigned long long *cnt, long long cap, int *ci, int *c
             h[0] = r.x;
             h[1] = r.y;
             h[2] = r.z;
-            const float4 vj = d.vstar[j], wi = d.wstar[i], wj = d.wstar[j];
-            const float ri = xi.w, rj = d.pos[j].w;
+            const float4 wi = d.wstar[i], wj = d.wstar[j];
+            const float ri = xi.w, rj = xj.w;
             const float sx = __fadd_rn(__fmul_rn(ri, wi.x), __fmul_rn(rj, wj.x));
             const float sy = __fadd_rn(__fmul_rn(ri, wi.y), __fmul_rn(rj, wj.y));
             const float sz = __fadd_rn(__fmul_rn(ri, wi.z), __fmul_rn(rj, wj.z));
@@ -416,7 +659,6 @@ k_contact_list(DemDev d, unsigned long long *cnt, long long cap, int *ci, int *c
                 __fsub_rn(__fsub_rn(vi.y, vj.y), __fsub_rn(__fmul_rn(sz, n[0]), __fmul_rn(sx, n[2]))),
                 __fsub_rn(__fsub_rn(vi.z, vj.z), __fsub_rn(__fmul_rn(sx, n[1]), __fmul_rn(sy, n[0])))};
             const float un = dot_rn(u[0], u[1], u[2], n);
-            const float meff = 1.0f / (vi.w + vj.w);
             const float gt =
                 __fmul_rn(d.gt_ratio, __fmul_rn(d.two_zeta, __fsqrt_rn(__fmul_rn(meff, d.kn))));
             for (int c = 0; c < 3; ++c)
@@ -475,12 +717,13 @@ __global__ void k_restore_im(DemDev d)
 
 struct dem_ctx {
     DemDev d{};
+    DemBuffers b{};
     dem_params prm{};
     lvb_ctx *bp = nullptr;
     cudaStream_t stream = nullptr;
-    cudaGraphExec_t graph = nullptr;
-    int64_t graph_steps = 0;
-    int graph_version = 0;
+    int advance_blocks = 0;      // launch shape of k_advance, worked out for
+    int advance_threads = 0;     // the broad phase's step_version shape_of
+    int shape_of = -1;
 };
 
 namespace {
@@ -496,10 +739,9 @@ int grid_n(int n) { return (n + kThreads - 1) / kThreads; }
 
 void dem_free(dem_ctx *c)
 {
-    if (c->graph) cudaGraphExecDestroy(c->graph);
     if (c->bp) lvb_destroy(c->bp);
     float4 *ptrs[] = {c->d.pos, c->d.vel, c->d.acc, c->d.vstar, c->d.omega, c->d.alpha,
-                      c->d.wstar};
+                      c->d.wstar, c->b.x[1], c->b.v[1], c->b.a[1], c->b.w[1], c->b.al[1]};
     for (float4 *p : ptrs)
         if (p) cudaFree(p);
 }
@@ -522,45 +764,51 @@ int launch_phase(dem_ctx *c, int phase)
                           (const float *)c->d.acc);
         if (rc) return rc;
     } else if (phase == DEM_PHASE_FORCES) {
-        k_forces<<<grid_n(c->d.n), kThreads, 0, c->stream>>>(c->d);
+        if (c->d.omega) k_forces<true><<<grid_n(c->d.n), kThreads, 0, c->stream>>>(c->d);
+        else k_forces<false><<<grid_n(c->d.n), kThreads, 0, c->stream>>>(c->d);
     } else {
         return LVB_EINVAL;
     }
     return from_cuda(cudaGetLastError());
 }
 
-// Launch shape of the fused step: the broad phase's block size, and no more
-// blocks than fit on the device at once for this kernel.
-int fused_shape(dem_ctx *c, dim3 *grid, dim3 *block)
+// Launch shape of k_advance: the broad phase's block size, as many blocks as
+// are resident on the device at once, and no more than have work.
+int advance_shape(dem_ctx *c)
 {
-    int blocks = 0, threads = 0, dev = 0, sms = 0, per_sm = 0;
-    step_shape(c->bp, &blocks, &threads);
+    const int version = step_version(c->bp);
+    if (c->shape_of == version) return LVB_OK;
+    int threads = 0, dev = 0, sms = 0, per_sm = 0;
+    step_shape(c->bp, nullptr, &threads);
+    const void *fn = c->d.omega ? (const void *)k_advance<true> : (const void *)k_advance<false>;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step<true, DemTail>, threads,
-                                                          0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0);
     if (e != cudaSuccess) return from_cuda(e);
     if (per_sm < 1) return LVB_EDEVICE;
-    *grid = dim3(std::min(blocks, per_sm * sms));
-    *block = dim3(threads);
+    // a run of up to 2,048 particles stays on one block, whose barriers cost
+    // next to nothing
+    const int want = c->d.n <= 2 * threads ? 1 : (c->d.n + threads - 1) / threads;
+    c->advance_blocks = std::min(want, per_sm * sms);
+    c->advance_threads = threads;
+    c->shape_of = version;
     return LVB_OK;
 }
 
-// One whole step (half-step, broad phase, forces) as one cooperative launch.
-int launch_fused(dem_ctx *c)
+// `steps` whole steps as one cooperative launch.
+int launch_advance(dem_ctx *c, int steps)
 {
     int rc = grow_stores_if_asked(c->bp);
     if (rc) return rc;
-    refresh(c);
-    dim3 grid, block;
-    rc = fused_shape(c, &grid, &block);
+    rc = advance_shape(c);
     if (rc) return rc;
-    const DemDev &d = c->d;
-    return from_cuda(launch_coop(k_step<true, DemTail>, grid, block, 0, c->stream,
-                                 (const float4 *)d.pos, (const float4 *)d.vstar,
-                                 (const float4 *)d.acc, step_state(c->bp), integrate_args(d),
-                                 DemTail{d}));
+    refresh(c);
+    const dim3 grid(c->advance_blocks), block(c->advance_threads);
+    return from_cuda(c->d.omega ? launch_coop(k_advance<true>, grid, block, 0, c->stream,
+                                              step_state(c->bp), c->d, c->b, steps)
+                                : launch_coop(k_advance<false>, grid, block, 0, c->stream,
+                                              step_state(c->bp), c->d, c->b, steps));
 }
 
 }  // namespace
@@ -612,16 +860,26 @@ static int dem_init_impl(dem_ctx **out, int32_t n_scenes, const int64_t *offsets
     if (e == cudaSuccess) e = cudaMalloc((void **)&d.vel, sizeof(float4) * n);
     if (e == cudaSuccess) e = cudaMalloc((void **)&d.acc, sizeof(float4) * n);
     if (e == cudaSuccess) e = cudaMalloc((void **)&d.vstar, sizeof(float4) * n);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.x[1], sizeof(float4) * n);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.v[1], sizeof(float4) * n);
+    if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.a[1], sizeof(float4) * n);
     if (prm->mu > 0.0f) {
         if (e == cudaSuccess) e = cudaMalloc((void **)&d.omega, sizeof(float4) * n);
         if (e == cudaSuccess) e = cudaMalloc((void **)&d.alpha, sizeof(float4) * n);
         if (e == cudaSuccess) e = cudaMalloc((void **)&d.wstar, sizeof(float4) * n);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.w[1], sizeof(float4) * n);
+        if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.al[1], sizeof(float4) * n);
     }
     if (e != cudaSuccess) {
         dem_free(c);
         delete c;
         return from_cuda(e);
     }
+    c->b.x[0] = d.pos;
+    c->b.v[0] = d.vel;
+    c->b.a[0] = d.acc;
+    c->b.w[0] = d.omega;
+    c->b.al[0] = d.alpha;
     k_dem_setup<<<std::min(grid_n((int)n), 4 * kNumSMs), kThreads, 0, c->stream>>>(
         d, (const float4 *)pos_r, (const float4 *)vel, prm->rho);
     int rc = offsets ? lvb_batch_init(&c->bp, n_scenes, offsets, (const float *)d.pos, box, skin,
@@ -650,7 +908,7 @@ static int dem_init_impl(dem_ctx **out, int32_t n_scenes, const int64_t *offsets
     DemDev d0 = d;
     d0.half_dt = 0.0f;
     d0.omega = d0.alpha = d0.wstar = nullptr;
-    k_forces<<<grid_n(d.n), kThreads, 0, c->stream>>>(d0);
+    k_forces<false><<<grid_n(d.n), kThreads, 0, c->stream>>>(d0);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
@@ -691,51 +949,16 @@ int dem_advance(dem_ctx *c, int64_t steps)
 {
     if (!c || steps < 0) return LVB_EINVAL;
     cudaGetLastError();   // clear a stale error of an unrelated earlier call
-    const int64_t chunk = DEM_GRAPH_STEPS;
-    int64_t done = 0;
-    while (steps - done >= chunk) {
-        // a store asked to grow: grow it (the graph holds the old store's
-        // addresses, so it is rebuilt below)
-        int rc = grow_stores_if_asked(c->bp);
+    // mirrored velocities cannot be worked out again from v and a, as a
+    // pass over several steps does for a contact's partner: with specular
+    // walls and contacts every step is a launch of its own
+    const bool single = c->d.wall_kind == DEM_WALL_SPECULAR && c->d.contacts_on;
+    const int64_t most = single ? 1 : DEM_GRAPH_STEPS;
+    for (int64_t done = 0; done < steps;) {
+        const int64_t m = std::min(most, steps - done);
+        const int rc = launch_advance(c, (int)m);
         if (rc) return rc;
-        if (c->graph && c->graph_version != graph_version(c->bp)) {
-            cudaGraphExecDestroy(c->graph);
-            c->graph = nullptr;
-        }
-        if (!c->graph) {
-            // one graph of `chunk` cooperative step kernels, built node by
-            // node (no stream capture, so any stream works, the legacy
-            // default one included)
-            refresh(c);
-            dim3 grid, block;
-            rc = fused_shape(c, &grid, &block);
-            if (rc) return rc;
-            const DemDev &d = c->d;
-            const DevState st = step_state(c->bp);
-            const IntegrateArgs ia = integrate_args(d);
-            cudaGraph_t g = nullptr;
-            cudaError_t e = cudaGraphCreate(&g, 0);
-            cudaGraphNode_t dep = nullptr;
-            for (int64_t k = 0; k < chunk && e == cudaSuccess; ++k)
-                e = add_coop_kernel(&dep, g, &dep, k_step<true, DemTail>, grid, block,
-                                    (const float4 *)d.pos, (const float4 *)d.vstar,
-                                    (const float4 *)d.acc, st, ia, DemTail{d});
-            if (e == cudaSuccess) e = cudaGraphInstantiate(&c->graph, g, 0);
-            if (g) cudaGraphDestroy(g);
-            if (e != cudaSuccess) {
-                c->graph = nullptr;
-                return from_cuda(e);
-            }
-            c->graph_steps = chunk;
-            c->graph_version = graph_version(c->bp);
-        }
-        const cudaError_t e = cudaGraphLaunch(c->graph, c->stream);
-        if (e != cudaSuccess) return from_cuda(e);
-        done += chunk;
-    }
-    for (; done < steps; ++done) {
-        const int rc = launch_fused(c);
-        if (rc) return rc;
+        done += m;
     }
     return LVB_OK;
 }

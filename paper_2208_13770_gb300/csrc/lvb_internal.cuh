@@ -19,8 +19,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-#include <tuple>
-
 #include "lvb.h"
 #include "lvb_mlp.h"
 
@@ -40,14 +38,15 @@ enum TraceSlot {
 
 struct DevCounters {
     int nF;            // flagged at the last step (final)
-    int nF_acc[2];     // flagged count while the check runs (slot: step parity)
-    int ovf[2];        // a row outgrew its capacity (slot: step parity)
+    int nF_acc[3];     // flagged count while the check runs (slot: step_slot)
+    int nE_acc[3];     // updated early beyond them (LVB_OPT_EARLY)
+    int ovf[3];        // a row outgrew its capacity (slot: step_slot)
     int row_overflow;  // same, for the separate full-build kernels
     int force_relayout;  // the next step that rebuilds rows re-lays them out (test hook)
     unsigned err;      // sticky DERR_* bits
     int last_flagged;
     int last_updated;
-    unsigned long long bar_cnt[2];  // grid-barrier arrivals in the step kernel, by step parity
+    unsigned long long bar_cnt[3];  // grid-barrier arrivals in the step kernel (slot: step_slot)
     long long steps;
     long long rebuild_steps;
     long long flagged_total;
@@ -244,10 +243,14 @@ __device__ __forceinline__ float mlp_skin(const lvb_mlp_weights *__restrict__ W,
 
 // Slack rule of the row store: capacity for a row of `len` entries (room
 // for the row to grow by half, and by 8 however short it is, before the
-// store is re-laid out).
+// store is re-laid out).  Every row's capacity, with slack or without, is a
+// multiple of four, so that every row starts on a 16-byte boundary and is
+// read four entries at a time (entries past the row's length hold -1).
+__host__ __device__ __forceinline__ int row_tight(int len) { return (len + 3) & ~3; }
+
 __host__ __device__ __forceinline__ int row_capacity(int len)
 {
-    return len + 8 + (len >> 1);
+    return row_tight(len + 8 + (len >> 1));
 }
 
 }  // namespace lvb
@@ -256,58 +259,40 @@ __host__ __device__ __forceinline__ int row_capacity(int len)
 // driver in the same library; not part of the C-ABI).
 namespace lvb {
 // Velocity-Verlet position half-step of the DEM driver, shared by its own
-// integrate kernel and by the check kernel that fuses it (identical
+// integrate kernel and by the kernel that advances whole steps (identical
 // arithmetic either way: explicit roundings, no compiler-chosen fusion):
 //   x' = x + (v dt + a dt^2/2),  v* = v + a dt   (v*.w keeps 1/m)
 // with specular reflection at the scene box when `specular` (x mirrored, v
-// and v* negated per axis).
-struct IntegrateArgs {
-    float4 *pos, *vel, *acc, *vstar;
-    float4 *omega, *alpha, *wstar;   // rotation (friction), or null
-    float dt, half_dt2;
-    int specular;
-    int active;     // 0: the check reads positions as they are
-};
-
-// kStream (the integrator as a kernel of its own): the old state is read
-// with streaming loads (evict first), so that the L2 keeps the new
-// positions this kernel writes for the broad phase that follows; inside the
-// fused step (kStream false) the forces tail reads v and a again.
-template <bool kStream = false>
-__device__ __forceinline__ float4 integrate_one(const IntegrateArgs &a, const SceneGeom &g, int i)
+// and v* negated per axis; returns true if v may have changed).
+__device__ __forceinline__ float4 star_of(float4 v, float4 ac, float dt)
 {
-    float4 x = kStream ? __ldcs(a.pos + i) : a.pos[i];
-    float4 v = kStream ? __ldcs(a.vel + i) : a.vel[i];
-    const float4 ac = kStream ? __ldcs(a.acc + i) : a.acc[i];
-    const float im = v.w;   // the driver keeps 1 / m in v.w (and v*.w)
-    x.x = __fadd_rn(x.x, fmaf(ac.x, a.half_dt2, __fmul_rn(v.x, a.dt)));
-    x.y = __fadd_rn(x.y, fmaf(ac.y, a.half_dt2, __fmul_rn(v.y, a.dt)));
-    x.z = __fadd_rn(x.z, fmaf(ac.z, a.half_dt2, __fmul_rn(v.z, a.dt)));
-    float4 vs = make_float4(fmaf(ac.x, a.dt, v.x), fmaf(ac.y, a.dt, v.y), fmaf(ac.z, a.dt, v.z), im);
-    if (a.specular) {
-        const float r = x.w;
-        float lo = __fadd_rn(g.lo[0], r), hi = __fsub_rn(g.hi[0], r);
-        if (x.x < lo || x.x > hi) {
-            x.x = __fsub_rn(__fmul_rn(2.0f, x.x < lo ? lo : hi), x.x); v.x = -v.x; vs.x = -vs.x;
-        }
-        lo = __fadd_rn(g.lo[1], r); hi = __fsub_rn(g.hi[1], r);
-        if (x.y < lo || x.y > hi) {
-            x.y = __fsub_rn(__fmul_rn(2.0f, x.y < lo ? lo : hi), x.y); v.y = -v.y; vs.y = -vs.y;
-        }
-        lo = __fadd_rn(g.lo[2], r); hi = __fsub_rn(g.hi[2], r);
-        if (x.z < lo || x.z > hi) {
-            x.z = __fsub_rn(__fmul_rn(2.0f, x.z < lo ? lo : hi), x.z); v.z = -v.z; vs.z = -vs.z;
-        }
-        a.vel[i] = v;
+    return make_float4(fmaf(ac.x, dt, v.x), fmaf(ac.y, dt, v.y), fmaf(ac.z, dt, v.z), v.w);
+}
+
+__device__ __forceinline__ void half_step(float4 &x, float4 &v, float4 ac, float4 &vs, float dt,
+                                          float half_dt2)
+{
+    x.x = __fadd_rn(x.x, fmaf(ac.x, half_dt2, __fmul_rn(v.x, dt)));
+    x.y = __fadd_rn(x.y, fmaf(ac.y, half_dt2, __fmul_rn(v.y, dt)));
+    x.z = __fadd_rn(x.z, fmaf(ac.z, half_dt2, __fmul_rn(v.z, dt)));
+    vs = star_of(v, ac, dt);
+}
+
+__device__ __forceinline__ void reflect(float4 &x, float4 &v, float4 &vs, const SceneGeom &g)
+{
+    const float r = x.w;
+    float lo = __fadd_rn(g.lo[0], r), hi = __fsub_rn(g.hi[0], r);
+    if (x.x < lo || x.x > hi) {
+        x.x = __fsub_rn(__fmul_rn(2.0f, x.x < lo ? lo : hi), x.x); v.x = -v.x; vs.x = -vs.x;
     }
-    a.pos[i] = x;
-    a.vstar[i] = vs;
-    if (a.omega) {   // w* = w + al dt (w*.w keeps 1/I)
-        const float4 w = a.omega[i], al = a.alpha[i];
-        a.wstar[i] = make_float4(fmaf(al.x, a.dt, w.x), fmaf(al.y, a.dt, w.y),
-                                 fmaf(al.z, a.dt, w.z), w.w);
+    lo = __fadd_rn(g.lo[1], r); hi = __fsub_rn(g.hi[1], r);
+    if (x.y < lo || x.y > hi) {
+        x.y = __fsub_rn(__fmul_rn(2.0f, x.y < lo ? lo : hi), x.y); v.y = -v.y; vs.y = -vs.y;
     }
-    return x;
+    lo = __fadd_rn(g.lo[2], r); hi = __fsub_rn(g.hi[2], r);
+    if (x.z < lo || x.z > hi) {
+        x.z = __fsub_rn(__fmul_rn(2.0f, x.z < lo ? lo : hi), x.z); v.z = -v.z; vs.z = -vs.z;
+    }
 }
 
 struct DevState;
@@ -338,31 +323,13 @@ cudaStream_t step_stream(lvb_ctx *c);
 // word), used on its stream by calls that synchronise before returning.
 void small_scratch(lvb_ctx *c, unsigned **u32, unsigned long long **u64);
 
-// Changes whenever the step kernel's arguments change (options, logging,
-// store growth), so that a caller holding a graph of steps knows to rebuild
-// it.
-int graph_version(lvb_ctx *c);
+// Changes whenever the step kernel's arguments or launch shape change
+// (options, logging, store growth), so that a caller that keeps a launch
+// shape knows to work it out again.
+int step_version(lvb_ctx *c);
 
 // Grows the row store / cell slots if a kernel asked for it (see lvb_step).
 int grow_stores_if_asked(lvb_ctx *c);
-
-// Adds a kernel node running fn(args...) after the given dependency (none
-// when dep or *dep is null); the argument values are copied into the node.
-// add_coop_kernel adds a cooperative one (all blocks resident at once).
-template <typename... P, typename... A>
-cudaError_t add_kernel(cudaGraphNode_t *out, cudaGraph_t g, const cudaGraphNode_t *dep,
-                       void (*fn)(P...), dim3 grid, dim3 block, A... args);
-
-template <typename... P, typename... A>
-cudaError_t add_coop_kernel(cudaGraphNode_t *out, cudaGraph_t g, const cudaGraphNode_t *dep,
-                            void (*fn)(P...), dim3 grid, dim3 block, A... args)
-{
-    cudaError_t e = add_kernel(out, g, dep, fn, grid, block, args...);
-    if (e != cudaSuccess) return e;
-    cudaLaunchAttributeValue v = {};
-    v.cooperative = 1;
-    return cudaGraphKernelNodeSetAttribute(*out, cudaLaunchAttributeCooperative, &v);
-}
 
 // Launches fn(args...) cooperatively on `stream` with `smem` bytes of
 // dynamic shared memory.
@@ -384,24 +351,4 @@ cudaError_t launch_coop(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cu
     return cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
 }
 
-template <typename... P, typename... A>
-cudaError_t add_kernel(cudaGraphNode_t *out, cudaGraph_t g, const cudaGraphNode_t *dep,
-                       void (*fn)(P...), dim3 grid, dim3 block, A... args)
-{
-    static_assert(sizeof...(P) == sizeof...(A), "argument count");
-    std::tuple<P...> vals(args...);
-    void *ptrs[sizeof...(P) > 0 ? sizeof...(P) : 1];
-    std::apply([&](auto &...v) {
-        int k = 0;
-        ((ptrs[k++] = (void *)&v), ...);
-    }, vals);
-    cudaKernelNodeParams p = {};
-    p.func = (void *)fn;
-    p.gridDim = grid;
-    p.blockDim = block;
-    p.sharedMemBytes = 0;
-    p.kernelParams = ptrs;
-    p.extra = nullptr;
-    return cudaGraphAddKernelNode(out, g, dep && *dep ? dep : nullptr, dep && *dep ? 1 : 0, &p);
-}
 }  // namespace lvb

@@ -21,10 +21,9 @@
 //              states, cells and rows of every particle
 //   -- barrier --
 //   re-layout  only if a row overflowed in the rebuild
-//   tail       the DEM driver's forces (k_step instantiated by lvb_dem.cu)
 // A step with nothing flagged is the check and one barrier.  The kernel is
-// included by lvb_broad.cu (the broad phase alone) and lvb_dem.cu (a whole
-// DEM step per launch).
+// included by lvb_broad.cu (the broad phase alone); lvb_dem.cu runs the same
+// phases after its own check pass, many DEM steps to a launch (k_advance).
 #pragma once
 
 #include "lvb_internal.cuh"
@@ -32,7 +31,8 @@
 namespace lvb {
 
 constexpr int kStepMaxThreads = 1024;     // block size limit of k_step (one block per SM)
-constexpr int kCheckUnroll = 2;           // 32-particle chunks a warp has in flight
+constexpr int kCheckUnroll = 2;           // chunks of 32 particles a warp of the step kernel
+                                          // should find at least (sizes its grid)
 constexpr int kFlaggedDirectMax = 4096;   // default of DevState::direct_max
 constexpr int kDirectUnroll = 4;          // flagged reference states per lane in flight
 constexpr unsigned kBarrierSpins = 1u << 22;   // ~1-3 s of polling (L2 round trips) before a barrier gives up
@@ -60,9 +60,9 @@ struct DevState {
     float4 *fref;     // their new (xref, R_NL), same order
     float4 *oref;     // their old (xref, R_NL), same order
     // many scenes: the flagged particles of scene q also sit in its own
-    // segment [first_q, first_q + sc_cnt[par][q]) of sfid / sfref, so the
+    // segment [first_q, first_q + sc_cnt[slot][q]) of sfid / sfref, so the
     // direct flagged test scans only its scene (null with one scene)
-    int *sc_cnt;      // 2 x nscenes counters (by step parity)
+    int *sc_cnt;      // 3 x nscenes counters (by step_slot)
     int *sfid;
     float4 *sfref;
     int *fsc;         // scene of each flagged particle, same order as fid
@@ -127,6 +127,15 @@ struct DevState {
 
 // gate modes of the separate full-build kernels (init, store growth)
 enum Gate { GATE_OVERFLOW = 1, GATE_ANY_FLAG = 2, GATE_ALWAYS = 3 };
+
+// Per-step counts live in three slots, step_slot(step) at a step: the steps
+// of one kernel follow one another with as little as one grid barrier
+// between them, so a block may already count the next step while another
+// still reads this one's counts, and only the slot of the step before is
+// free for everyone.  Each step clears that one after its first barrier,
+// which is the slot of the step after the next.
+__device__ __forceinline__ int step_slot(int step) { return step % 3; }
+__device__ __forceinline__ int spent_slot(int slot) { return slot == 0 ? 2 : slot - 1; }
 
 __device__ __forceinline__ const SceneGeom &geom_of(const DevState &s, int i)
 {
@@ -316,7 +325,7 @@ __device__ __forceinline__ void update_group(const DevState &s, const lvb_mlp_we
     if (s.sc_cnt) {
         const int sc = s.scene_of[i];
         s.fsc[k] = sc;
-        const int slot = g.first + atomicAdd(&s.sc_cnt[(step & 1) * s.nscenes + sc], 1);
+        const int slot = g.first + atomicAdd(&s.sc_cnt[step_slot(step) * s.nscenes + sc], 1);
         s.sfid[slot] = i;
         s.sfref[slot] = qn;
     }
@@ -355,7 +364,7 @@ static __device__ __noinline__ void update_lanes(const DevState &s, const int *i
     if (s.sc_cnt) {
         const int sc = s.scene_of[i];
         s.fsc[k] = sc;
-        const int slot = g.first + atomicAdd(&s.sc_cnt[(step & 1) * s.nscenes + sc], 1);
+        const int slot = g.first + atomicAdd(&s.sc_cnt[step_slot(step) * s.nscenes + sc], 1);
         s.sfid[slot] = i;
         s.sfref[slot] = qn;
     }
@@ -575,7 +584,7 @@ __device__ __forceinline__ void lane_edit(const DevState &s, int jr, int ji, int
 // The edits of other rows run one per lane, in parallel; the first 32 old
 // partners and the first 32 stencil candidates are loaded together.
 static __device__ __noinline__ void patch_warp(const DevState &s, int k, int nF, bool direct,
-                                               int par, int *ovf, unsigned (&work)[3])
+                                               int slot, int *ovf, unsigned (&work)[3])
 {
     const int lane = threadIdx.x & 31;
     const unsigned lt = lanemask_lt();
@@ -587,7 +596,7 @@ static __device__ __noinline__ void patch_warp(const DevState &s, int k, int nF,
     const SceneGeom &g = s.sg[sc];
     // the direct test's count, loaded now (its latency under the stencil's)
     const bool own = s.sc_cnt != nullptr;
-    const int m_dir = !direct ? 0 : own ? s.sc_cnt[par * s.nscenes + sc] : nF;
+    const int m_dir = !direct ? 0 : own ? s.sc_cnt[slot * s.nscenes + sc] : nF;
     const int d0 = g.dim[0], d1 = g.dim[1], d2 = g.dim[2];
     const int ci = cell_key(g, qn.x, qn.y, qn.z) - g.cell_base;
     const int cx = ci % d0, cy = (ci / d0) % d1, cz = ci / (d0 * d1);
@@ -773,7 +782,7 @@ __device__ __forceinline__ void own_row_insert(const DevState &s, int off, int c
 //      of a flagged partner is kept in pold) joins row i with zero
 //      history, and an unflagged partner gets i in its row.
 static __device__ __noinline__ void patch_warp_hist(const DevState &s, int k, int nF, bool direct,
-                                                    int par, int *ovf, unsigned (&work)[3])
+                                                    int slot, int *ovf, unsigned (&work)[3])
 {
     const int lane = threadIdx.x & 31;
     const int ccap = s.ccap;
@@ -852,7 +861,7 @@ static __device__ __noinline__ void patch_warp_hist(const DevState &s, int k, in
         const bool own = s.sc_cnt != nullptr;
         const float4 *lst = own ? s.sfref + g.first : s.fref;
         const int *ids = own ? s.sfid + g.first : s.fid;
-        const int m = own ? s.sc_cnt[par * s.nscenes + sc] : nF;
+        const int m = own ? s.sc_cnt[slot * s.nscenes + sc] : nF;
         work[1] += m;
         for (int b0 = 0; b0 < m; b0 += 32) {
             const int kk = b0 + lane;
@@ -960,16 +969,18 @@ __device__ __forceinline__ void ph_rows(const DevState &s, int nitems, int fill,
 }
 
 // ---------------------------------------------------------------------------
-// Grid-wide barrier of the step kernel (all blocks co-resident).  A 64-bit
-// arrival counter per step parity: the kernel of a step counts on
-// bar_cnt[parity] (which starts at zero) and clears the other one for the
-// next step.  Thread 0 of each block arrives with a release add (no
+// Grid-wide barrier of the step kernels (all blocks co-resident).  A 64-bit
+// arrival counter per step slot: a step counts on bar_cnt[slot] (which
+// starts at zero).  Thread 0 of each block arrives with a release add (no
 // return value to wait for) and polls with acquire loads until the counter
-// holds the arrivals of this barrier and of all earlier ones in the kernel.
+// holds the arrivals of this barrier and of all earlier ones of the step.
 // Polling is bounded: after s.bar_spins polls (kBarrierSpins unless a test
 // lowers it) the block records DERR_SYNC and leaves; every block then
 // returns, and later steps do nothing (the context reports LVB_ETIMEOUT).
 // Returns false when the step must be abandoned.
+// A grid of one block (up to 2,048 particles) needs the block barrier only:
+// on the 2,000-sphere ballistic run the arrival and the polls through L2
+// would be most of a step without flags.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void red_add_release(unsigned long long *p, unsigned long long v)
 {
@@ -985,26 +996,33 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
 
 // the barrier state of this block (used by its thread 0 only)
 static __shared__ unsigned long long s_bar_need;   // arrivals up to the last barrier
-static __shared__ int s_bar_par;                   // parity of the step
-// the block's share of the partial rebuild's work counts (DevCounters
+static __shared__ int s_bar_slot;                  // slot of the step
+// the block's share of the partial rebuilds' work counts (DevCounters
 // alg_*), gathered by its warps with shared-memory atomics and added to the
-// context's counters by thread 0 once per step
+// context's counters by thread 0 once per kernel
 static __shared__ unsigned long long s_work[3];
 // the block's rebuild work items when traced: first start, last end,
 // longest item (item_start / item_stop)
 static __shared__ unsigned long long s_items[3];
 static __shared__ unsigned long long s_item_t0[kStepMaxThreads / 32];
 
-// Called by every thread at the start of the step kernel, before any barrier.
-__device__ __forceinline__ void grid_barrier_begin(const DevState &s, int par)
+// Called by every thread at the start of a step kernel, before any barrier
+// (whose block barrier publishes what is set here).
+__device__ __forceinline__ void step_kernel_begin()
 {
     if (threadIdx.x == 0) {
-        s_bar_need = 0;
-        s_bar_par = par;
         s_work[0] = s_work[1] = s_work[2] = 0ULL;
         s_items[0] = ~0ULL;
         s_items[1] = s_items[2] = 0ULL;
-        if (blockIdx.x == 0) s.cnt->bar_cnt[par ^ 1] = 0;
+    }
+}
+
+// Called by every thread at the start of a step, before its first barrier.
+__device__ __forceinline__ void grid_barrier_begin(int slot)
+{
+    if (threadIdx.x == 0) {
+        s_bar_need = 0;
+        s_bar_slot = slot;
     }
 }
 
@@ -1012,9 +1030,13 @@ __device__ __forceinline__ bool grid_barrier(const DevState &s)
 {
     __shared__ int s_ok;
     __syncthreads();
+    if (gridDim.x == 1 && s.bar_extra == 0) {
+        if (threadIdx.x == 0) atomicAdd(&s.cnt->barriers, 1ULL);
+        return true;
+    }
     if (threadIdx.x == 0) {
         DevCounters *c = s.cnt;
-        unsigned long long *w = &c->bar_cnt[s_bar_par];
+        unsigned long long *w = &c->bar_cnt[s_bar_slot];
         const unsigned long long need = s_bar_need + gridDim.x + s.bar_extra;
         s_bar_need = need;
         red_add_release(w, 1ULL);
@@ -1169,47 +1191,6 @@ __device__ __forceinline__ void flag_chunks(const DevState &s, const int (&cu)[U
         if (b >> lane & 1u) pd.id[pd.n + __popc(b & lt)] = cu[u] + lane;
         pd.n += __popc(b);
     }
-}
-
-// The check pass of the DEM form: each thread first performs the driver's
-// position half-step of its particles (integrate_one), so the positions are
-// produced here and read back from registers.  Block b takes tiles b,
-// b + grid, ... of blockDim * kCheckUnroll particles; in a tile each warp
-// checks kCheckUnroll chunks of 32 (loads of all chunks first).
-__device__ __forceinline__ void check_pass_fused(const DevState &s, const float4 *vel,
-                                                 const float4 *acc, const IntegrateArgs &ia,
-                                                 bool inc, int step, int *nF_acc)
-{
-    __shared__ int pend_id[kStepMaxThreads / 32][kPending];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    Pending pd{pend_id[warp], 0};
-    const int tile = blockDim.x * kCheckUnroll;
-    for (int t0 = blockIdx.x * tile; t0 < s.n; t0 += gridDim.x * tile) {
-        float4 p[kCheckUnroll], q[kCheckUnroll];
-        int cu[kCheckUnroll];
-        bool f[kCheckUnroll];
-#pragma unroll
-        for (int u = 0; u < kCheckUnroll; ++u) {
-            cu[u] = t0 + u * blockDim.x + warp * 32;
-            const int i = cu[u] + lane;
-            if (i < s.n) {
-                p[u] = integrate_one(ia, geom_of(s, i), i);
-                q[u] = s.ref[i];
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kCheckUnroll; ++u) {
-            const int i = cu[u] + lane;
-            f[u] = false;
-            if (i < s.n) {
-                f[u] = violates(p[u], q[u]);
-                if (!(isfinite(p[u].x) && isfinite(p[u].y) && isfinite(p[u].z)))
-                    atomicOr(&s.cnt->err, DERR_NAN);
-            }
-        }
-        flag_chunks<kCheckUnroll>(s, cu, f, ia.pos, vel, acc, inc, step, nF_acc, pd);
-    }
-    flush_pending_final(s, pd, ia.pos, vel, acc, inc, step, nF_acc);
 }
 
 // The check pass of the broad phase alone, register form
@@ -1462,7 +1443,7 @@ static __device__ __noinline__ void save_rows_pass(const DevState &s)
 }
 
 // Offsets of the row store by a grid-wide exclusive scan of the row sizes
-// (row_capacity(len), or len itself when tight), block b owning rows
+// (row_capacity(len), or row_tight(len) when tight), block b owning rows
 // [b * per, (b + 1) * per); block 0 scans the block sums and writes the
 // total to store_needed.  Every block returns the total (read after a
 // barrier).  Returns -1 when the step must be abandoned.
@@ -1474,7 +1455,7 @@ static __device__ long long layout_scan(const DevState &s, bool tight)
     const int hi = (int)min((long long)s.n, lo + per);
     long long sum = 0, tot;
     for (int i = lo + threadIdx.x; i < hi; i += blockDim.x)
-        sum += tight ? s.row_len[i] : row_capacity(s.row_len[i]);
+        sum += tight ? row_tight(s.row_len[i]) : row_capacity(s.row_len[i]);
     block_scan_any(sum, &tot);
     if (threadIdx.x == 0) s.blk[blockIdx.x] = tot;
     if (!grid_barrier(s)) return -1;
@@ -1497,7 +1478,8 @@ static __device__ long long layout_scan(const DevState &s, bool tight)
     long long run = s.blk[blockIdx.x];
     for (int i0 = lo; i0 < hi; i0 += blockDim.x) {
         const int i = i0 + threadIdx.x;
-        const int v = i < hi ? (tight ? s.row_len[i] : row_capacity(s.row_len[i])) : 0;
+        const int v =
+            i < hi ? (tight ? row_tight(s.row_len[i]) : row_capacity(s.row_len[i])) : 0;
         const long long ex = block_scan_any(v, &tot);
         if (i < hi) {
             s.row_off[i] = (int)min(run + ex, (long long)INT32_MAX);
@@ -1588,10 +1570,12 @@ static __device__ __noinline__ void log_pass(const DevState &s, const float4 *po
 // reading of Def. autoverlet's trigger between its per-particle and global
 // forms: the pair set stays the function of (xref, skin) it always is).
 // One warp per 32 consecutive particles: the updated-set word ubits = the
-// flag word | the early ones; the early ones join the flagged list (one
-// atomic per warp) and, unless the update is deferred, are updated here.
+// flag word | the early ones; the early ones join the flagged list behind
+// the nV violations (one atomic per warp, on a counter of their own: other
+// blocks may still be reading the violations') and, unless the update is
+// deferred, are updated here.
 static __device__ __noinline__ void early_pass(const DevState &s, const float4 *pos,
-                                               const float4 *vel, int step, int *nF_acc)
+                                               const float4 *vel, int step, int nV, int *nE_acc)
 {
     const int lane = threadIdx.x & 31;
     const int w0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -1612,7 +1596,7 @@ static __device__ __noinline__ void early_pass(const DevState &s, const float4 *
         if (lane == 0) s.ubits[w] = fw | m;
         if (!m) continue;
         int k0 = 0;
-        if (lane == 0) k0 = atomicAdd(nF_acc, __popc(m));
+        if (lane == 0) k0 = nV + atomicAdd(nE_acc, __popc(m));
         k0 = __shfl_sync(FULL, k0, 0);
         const int r = __popc(m & lanemask_lt());
         if (e) {
@@ -1624,12 +1608,6 @@ static __device__ __noinline__ void early_pass(const DevState &s, const float4 *
         __syncwarp();
     }
 }
-
-// Tail of a step that only does the broad phase.
-struct NoTail {
-    static constexpr bool kActive = false;
-    __device__ void operator()(int, int) const {}
-};
 
 __device__ __forceinline__ void trace_add(DevCounters *c, int slot, unsigned long long a,
                                           unsigned long long b)
@@ -1683,6 +1661,8 @@ __device__ __forceinline__ void items_flush(const DevState &s)
         atomicMax(&c->tr_end[TR_ITEMS], s_items[1]);
         atomicMin(&c->tr_start[TR_ITEM_MAX], 0ULL);
         atomicMax(&c->tr_end[TR_ITEM_MAX], s_items[2]);
+        s_items[0] = ~0ULL;   // for the kernel's next step
+        s_items[1] = s_items[2] = 0ULL;
     }
 }
 
@@ -1692,7 +1672,7 @@ __device__ __forceinline__ void items_flush(const DevState &s)
 // skip the flagged particles in the cells and test them directly); more:
 // the moves first and a barrier, then the patches on final cells.  Returns
 // false when the step must be abandoned.
-static __device__ __noinline__ bool partial_pass(const DevState &s, int nF, int par, int *ovf)
+static __device__ __noinline__ bool partial_pass(const DevState &s, int nF, int slot, int *ovf)
 {
     // work items go round the blocks first (item w to block w % grid), so
     // that a few flagged particles spread over all SMs instead of filling
@@ -1710,16 +1690,16 @@ static __device__ __noinline__ bool partial_pass(const DevState &s, int nF, int 
         if (!grid_barrier(s)) return false;
         for (int k = w0; k < nF; k += nw) {
             item_start(s);
-            if (s.hist) patch_warp_hist(s, k, nF, false, par, ovf, work);
-            else patch_warp(s, k, nF, false, par, ovf, work);
+            if (s.hist) patch_warp_hist(s, k, nF, false, slot, ovf, work);
+            else patch_warp(s, k, nF, false, slot, ovf, work);
             item_stop(s);
         }
     } else {
         for (int w = w0; w < 2 * nF; w += nw) {
             item_start(s);
             if (w < nF) {
-                if (s.hist) patch_warp_hist(s, w, nF, true, par, ovf, work);
-                else patch_warp(s, w, nF, true, par, ovf, work);
+                if (s.hist) patch_warp_hist(s, w, nF, true, slot, ovf, work);
+                else patch_warp(s, w, nF, true, slot, ovf, work);
             } else {
                 move_warp(s, s.fid[w - nF], s.fref[w - nF], flagged_scene(s, w - nF));
             }
@@ -1735,7 +1715,7 @@ static __device__ __noinline__ bool partial_pass(const DevState &s, int nF, int 
 }
 
 // Adds the block's rebuild work counts to the context's (thread 0, after a
-// block barrier that follows partial_pass).
+// block barrier that follows the kernel's last partial_pass).
 __device__ __forceinline__ void flush_work(const DevState &s)
 {
     if (threadIdx.x == 0) {
@@ -1746,60 +1726,43 @@ __device__ __forceinline__ void flush_work(const DevState &s)
     }
 }
 
-// ---------------------------------------------------------------------------
-// One step.  pos_in / vel / acc: the caller's positions, velocities (policy
-// input) and accelerations; with kFused the positions come from the DEM
-// half-step (ia) instead.  Launched cooperatively with every block resident.
-// Per-step counts live in two slots chosen by the step's parity, so that the
-// slots of the next step can be cleared while this one is read.  The list
-// is final when the kernel ends (and before the tail).
-// ---------------------------------------------------------------------------
-template <bool kFused, class Tail>
-__global__ void __launch_bounds__(kStepMaxThreads, 1)
-k_step(const float4 *__restrict__ pos_in, const float4 *vel, const float4 *acc,
-       const __grid_constant__ DevState sp,
-       IntegrateArgs ia, Tail tail)
+// The step's bookkeeping (counters, trace) runs on the last warp of block 0,
+// whose rebuild work items come last.
+__device__ __forceinline__ bool step_lead()
 {
-    // the context's state read in place from the parameter space (uniform
-    // reads through the constant cache; no copy at the start)
-    const DevState &s = sp;
-    DevCounters *c = s.cnt;
-    // the step's bookkeeping (counters, trace) runs on the last warp of
-    // block 0, whose rebuild work items come last
-    const bool lead = blockIdx.x == 0 && threadIdx.x == blockDim.x - 32;
-    const unsigned long long t0 = (s.trace && lead) ? global_ns() : 0ULL;
-    // every thread reads the counters it needs (one broadcast load each, no
-    // block barrier before the check's loads); they are stable while the
-    // check runs
-    const unsigned err = c->err;
-    if (err & DERR_SYNC) return;   // a barrier failed earlier: the context is unusable
-    const bool inc = s.trigger == LVB_TRIGGER_PARTIAL && !(err & DERR_STORE);
-    const int step = (int)c->steps + 1, par = step & 1;
-    __shared__ __align__(16) lvb_mlp_weights w_sh;
-    const bool net = s.skin_kind == LVB_SKIN_LEARNED;
-    if (net) weights_copy_async(&w_sh, s.mlp);
-    grid_barrier_begin(s, par);
-    const float4 *pos = kFused ? ia.pos : pos_in;
-    int *ovf = &c->ovf[par];
+    return blockIdx.x == 0 && threadIdx.x == blockDim.x - 32;
+}
 
-    if constexpr (kFused)
-        check_pass_fused(s, vel, acc, ia, inc, step, &c->nF_acc[par]);
-    else if (s.check_regs)
-        check_pass_regs(s, pos_in, vel, acc, inc, step, &c->nF_acc[par]);
-    else
-        check_pass_stream(s, pos_in, vel, acc, inc, step, &c->nF_acc[par]);
-    if (net) weights_copy_wait();
-    if (!grid_barrier(s)) return;
-    const int nV = *(volatile int *)&c->nF_acc[par];   // violations of Eq. update
-    int nF = nV;                                        // particles updated
-    if (inc && nV > 0 && s.early_beta < 1.0f) {
-        early_pass(s, pos, vel, step, &c->nF_acc[par]);
-        if (!grid_barrier(s)) return;
-        nF = *(volatile int *)&c->nF_acc[par];
+// Everything of a step after its check pass: the first barrier, the early
+// trigger, the bookkeeping, the deferred updates, the rebuild with its
+// barrier, the re-layout, the rebuild log.  pos / vel / acc: what the check
+// saw (vel and acc are read for updated particles only; with a trigger that
+// updates everyone, for all).  The list is final for every block when it
+// returns true; false: the step was abandoned.  t0: start of the check
+// (trace).
+__device__ __forceinline__ bool finish_step(const DevState &s, const lvb_mlp_weights *w_sh,
+                                            const float4 *pos, const float4 *vel,
+                                            const float4 *acc, bool inc, int step, int slot,
+                                            unsigned long long t0)
+{
+    DevCounters *c = s.cnt;
+    const bool lead = step_lead();
+    int *ovf = &c->ovf[slot];
+    const int spent = spent_slot(slot);
+    if (!grid_barrier(s)) return false;
+    const int nV = *(volatile int *)&c->nF_acc[slot];   // violations of Eq. update
+    int nF = nV;                                         // particles updated
+    if (blockIdx.x == 0) {   // the spent slot, which the step after the next counts on
+        if (threadIdx.x == 0) c->bar_cnt[spent] = 0;
+        if (s.sc_cnt)
+            for (int q = threadIdx.x; q < s.nscenes; q += blockDim.x)
+                s.sc_cnt[spent * s.nscenes + q] = 0;
     }
-    if (s.sc_cnt && blockIdx.x == 0)   // the next step's scene counters
-        for (int q = threadIdx.x; q < s.nscenes; q += blockDim.x)
-            s.sc_cnt[(par ^ 1) * s.nscenes + q] = 0;
+    if (inc && nV > 0 && s.early_beta < 1.0f) {
+        early_pass(s, pos, vel, step, nV, &c->nE_acc[slot]);
+        if (!grid_barrier(s)) return false;
+        nF = nV + *(volatile int *)&c->nE_acc[slot];
+    }
     int upd;
     if (s.trigger == LVB_TRIGGER_PARTIAL) upd = nF;
     else if (s.trigger == LVB_TRIGGER_GLOBAL) upd = nV ? s.n : 0;
@@ -1807,8 +1770,9 @@ k_step(const float4 *__restrict__ pos_in, const float4 *vel, const float4 *acc,
     unsigned long long t1 = 0;
     if (lead) {
         // stores and reductions only: no load on the step's last path
-        c->nF_acc[par ^ 1] = 0;
-        c->ovf[par ^ 1] = 0;
+        c->nF_acc[spent] = 0;
+        c->nE_acc[spent] = 0;
+        c->ovf[spent] = 0;
         c->nF = nV;
         if (s.nf_out) *s.nf_out = nV;
         c->last_flagged = nV;
@@ -1817,7 +1781,6 @@ k_step(const float4 *__restrict__ pos_in, const float4 *vel, const float4 *acc,
         atomicAdd((unsigned long long *)&c->flagged_total, (unsigned long long)nV);
         atomicAdd((unsigned long long *)&c->updated_total, (unsigned long long)upd);
         if (upd) atomicAdd((unsigned long long *)&c->rebuild_steps, 1ULL);
-        atomicAdd(&c->kernels, 1ULL);
         if (s.trace) {
             t1 = global_ns();
             trace_add(c, TR_CHECK, t0, t1);
@@ -1834,24 +1797,23 @@ k_step(const float4 *__restrict__ pos_in, const float4 *vel, const float4 *acc,
     if (inc) {
         if (nF > 0) {
             if (deferred_update(s)) {
-                update_pass(s, &w_sh, nF, pos, vel, acc, step);
-                if (!grid_barrier(s)) return;
+                update_pass(s, w_sh, nF, pos, vel, acc, step);
+                if (!grid_barrier(s)) return false;
             }
-            if (!partial_pass(s, nF, par, ovf)) return;
+            if (!partial_pass(s, nF, slot, ovf)) return false;
             if (s.trace) items_flush(s);
             changed = true;
         }
     } else if (upd > 0 && !store_failed(s)) {
         full_update_pass(s, pos, vel);
-        if (!grid_barrier(s)) return;
+        if (!grid_barrier(s)) return false;
         full_insert_pass(s);
-        if (!grid_barrier(s)) return;
+        if (!grid_barrier(s)) return false;
         all_rows_pass(s, 1, ovf);
         changed = true;
     }
     if (changed) {
-        if (!grid_barrier(s)) return;
-        flush_work(s);
+        if (!grid_barrier(s)) return false;
         unsigned long long t2 = 0;
         if (s.trace && lead) {
             t2 = global_ns();
@@ -1864,19 +1826,12 @@ k_step(const float4 *__restrict__ pos_in, const float4 *vel, const float4 *acc,
             }
         }
         if ((*(volatile int *)ovf || *(volatile int *)&c->force_relayout) && !store_failed(s)) {
-            if (!relayout_pass(s)) return;
+            if (!relayout_pass(s)) return false;
             if (s.trace && lead) trace_add(c, TR_RELAYOUT, t2, global_ns());
         }
     }
     if (s.log_on) log_pass(s, pos, step);
-    if (Tail::kActive) {
-        const unsigned long long t3 = (s.trace && lead) ? global_ns() : 0ULL;
-        tail(blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
-        if (s.trace) {
-            if (!grid_barrier(s)) return;
-            if (lead) trace_add(c, TR_TAIL, t3, global_ns());
-        }
-    }
+    return true;
 }
 
 }  // namespace lvb
