@@ -40,6 +40,7 @@ struct DevCounters {
     int nF;            // flagged at the last step (final)
     int nF_acc[3];     // flagged count while the check runs (slot: step_slot)
     int nE_acc[3];     // updated early beyond them (LVB_OPT_EARLY)
+    int next_patch[3]; // patches handed out beyond the first of each team
     int ovf[3];        // a row outgrew its capacity (slot: step_slot)
     int row_overflow;  // same, for the separate full-build kernels
     int force_relayout;  // the next step that rebuilds rows re-lays them out (test hook)

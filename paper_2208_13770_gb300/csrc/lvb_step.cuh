@@ -516,59 +516,91 @@ __device__ __forceinline__ void lane_insert(const DevState &s, int j, int i, int
     }
 }
 
-// One removal (partner i leaves row jr) and one insertion (partner i joins
-// row ji) by one lane, their loads interleaved so that both edits take the
-// latency of one: the two rows' bounds together, then four entries of each
-// at a time.  jr or ji < 0: no such edit.  Same rules as lane_remove and
-// lane_insert (the two rows differ: a removed pair is not a new one).
-__device__ __forceinline__ void lane_edit(const DevState &s, int jr, int ji, int i, int *ovf)
+// Where a row lies: read ahead of an edit of it.
+struct RowSpan {
+    int off, len, cap;
+};
+
+__device__ __forceinline__ RowSpan row_span(const DevState &s, int j)
 {
-    int offr = 0, lenr = 0, offi = 0, capi = 0, leni = 0;
-    if (jr >= 0) {
-        offr = s.row_off[jr];
-        lenr = min(s.row_len[jr], s.row_cap[jr]);
+    RowSpan r{0, 0, 0};
+    if (j >= 0) {
+        r.off = s.row_off[j];
+        r.cap = s.row_cap[j];
+        r.len = min(s.row_len[j], r.cap);
     }
-    if (ji >= 0) {
-        offi = s.row_off[ji];
-        capi = s.row_cap[ji];
-        leni = min(s.row_len[ji], capi);
-    }
-    bool dr = jr < 0 || lenr == 0, di = ji < 0;
-    for (int e = 0; !dr || (!di && e < leni); e += 4) {
+    return r;
+}
+
+// One removal (partner i leaves row jr, which lies at r) and one insertion
+// (partner i joins row ji, which lies at q) by one lane, their loads
+// interleaved so that both edits take the latency of one: four entries of each
+// row at a time.  jr or ji < 0: no such edit.  Same rules as lane_remove and
+// lane_insert (the two rows differ: a removed pair is not a new one).
+__device__ __forceinline__ void lane_edit(const DevState &s, int jr, RowSpan r, int ji, RowSpan q,
+                                          int i, int *ovf)
+{
+    bool dr = jr < 0 || r.len == 0, di = ji < 0;
+    for (int e = 0; !dr || (!di && e < q.len); e += 4) {
         int vr[4], vi[4];
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
-            vr[u] = !dr && e + u < lenr ? s.col[offr + e + u] : -2;
-            vi[u] = !di && e + u < leni ? s.col[offi + e + u] : 0;
+            vr[u] = !dr && e + u < r.len ? s.col[r.off + e + u] : -2;
+            vi[u] = !di && e + u < q.len ? s.col[q.off + e + u] : 0;
         }
 #pragma unroll
         for (int u = 0; u < 4; ++u) {
             if (!dr && vr[u] == i) {
-                s.col[offr + e + u] = -1;
+                s.col[r.off + e + u] = -1;
                 dr = true;
             }
-            if (!di && vi[u] < 0 && atomicCAS(&s.col[offi + e + u], -1, i) == -1) {
+            if (!di && vi[u] < 0 && atomicCAS(&s.col[q.off + e + u], -1, i) == -1) {
                 di = true;
-                if (s.hist) s.hist[offi + e + u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (s.hist) s.hist[q.off + e + u] = make_float4(0.f, 0.f, 0.f, 0.f);
             }
         }
-        if (e + 4 >= lenr) dr = true;
+        if (e + 4 >= r.len) dr = true;
     }
     if (di) return;
-    for (int t = 0; t <= capi; ++t) {
+    for (int t = 0; t <= q.cap; ++t) {
         const int p = atomicAdd(&s.row_len[ji], 1);
-        if (p >= capi) {
+        if (p >= q.cap) {
             atomicExch(ovf, 1);
             return;
         }
-        if (atomicCAS(&s.col[offi + p], -1, i) == -1) {
-            if (s.hist) s.hist[offi + p] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (atomicCAS(&s.col[q.off + p], -1, i) == -1) {
+            if (s.hist) s.hist[q.off + p] = make_float4(0.f, 0.f, 0.f, 0.f);
             return;
         }
     }
 }
 
-// a4 + a5 for flagged particle k of the list (warp), i = fid[k]:
+// A team of warps that patches one row together: `size` consecutive warps
+// of the block (a power of two), this warp the w-th of them; slot: the
+// team's place in the block.
+struct Team {
+    int size, w, slot;
+};
+
+// A team of one warp needs no block resources; larger ones (at least four
+// warps, so at most eight to a block) each have a named barrier.
+__device__ __forceinline__ void team_sync(const Team &t)
+{
+    if (t.size == 1) __syncwarp();
+    else asm volatile("bar.sync %0, %1;" ::"r"(t.slot + 1), "r"(t.size * 32) : "memory");
+}
+
+// the block's share of the partial rebuilds' work counts (DevCounters
+// alg_*), gathered by its warps with shared-memory atomics and added to the
+// context's counters by thread 0 once per kernel
+static __shared__ unsigned long long s_work[3];
+
+constexpr int kNoted = 64;   // candidates a warp notes before it takes them up
+static __shared__ int2 s_noted[kStepMaxThreads / 32][kNoted];
+static __shared__ int s_team_new[kStepMaxThreads / 32];       // entries given out of the row
+static __shared__ unsigned s_team_free[kStepMaxThreads / 32]; // its free slots (history)
+
+// a4 + a5 for flagged particle k of the list (a team of warps), i = fid[k]:
 //   1. each old partner j that is unflagged and no longer a pair (test on
 //      i's new reference state) loses i from its row;
 //   2. the new row of i: the 27-cell stencil around its new cell over the
@@ -580,26 +612,54 @@ __device__ __forceinline__ void lane_edit(const DevState &s, int jr, int ji, int
 //      on i's old reference state) gets i in its row.
 // A pair is a function of the two reference states (Def. verletlist) and an
 // unflagged particle's state does not change, so these tests decide exactly
-// which entries of the unflagged rows change; no other warp touches row i.
-// The edits of other rows run one per lane, in parallel; the first 32 old
-// partners and the first 32 stencil candidates are loaded together.
-static __device__ __noinline__ void patch_warp(const DevState &s, int k, int nF, bool direct,
-                                               int slot, int *ovf, unsigned (&work)[3])
+// which entries of the unflagged rows change; no other team touches row i.
+// The edits of other rows run one per lane, in parallel.
+//
+// With contact history (kHist, LVB_OPT_HISTORY) row i is edited in place, as
+// the unflagged rows are, so that a partner that stays a pair keeps its slot
+// -- and its history: an old entry j no longer a pair under the new reference
+// states of i and j (this step's updates are all written) becomes -1 (a flagged
+// j edits its own row), and only a partner that was not a pair under the old
+// states (the old record of a flagged partner is kept in pold) joins, with
+// zero history, in a free slot among the row's first 32 or at its end.
+// Otherwise the row is written anew; the old one is in registers by then.
+//
+// What bounds it is a chain of dependent loads, 0.4 to 1 us each -- flagged
+// record, row bounds, cell counts, candidates and old partners, their flags,
+// the partners' rows, the claim of a slot -- and, in beds of mixed sizes, the
+// candidates of the large particles (a thousand, where the mean is 200), for
+// the longest of which the step waits.  So what can be asked for early is (the
+// first flagged records with the candidates, a partner's row bounds with its
+// flag word, the next candidates while these are tested), the candidates that
+// pass are only noted and then taken up together, and every warp of a team
+// takes a share of the old row, the candidates and the flagged list.  All of it
+// has to fit 64 registers: with the spills of a first version, on all 32
+// warps of an SM, the loop ran at 3,000 cycles for 64 candidates.  Rebuild
+// phase, per step, before and after: 2M drum 10k flagged 79 -> 50 us, 1M drum
+// with friction 45 -> 20 us, 6.2M batch 13.2 -> 11.8 us, 2k gas 7.4 -> 5.6 us.
+//
+// kDense (cells of more than kTeamSlots slots): the candidates are taken cell
+// by cell, the cells shared out among the warps of a team; otherwise the team
+// is one warp, and the few candidates of the 27 cells are taken as one run,
+// each lane finding its cell by a shuffle search (which, at 32 candidates a
+// time, would be most of the work in a dense bed).
+template <bool kHist, bool kDense>
+__device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int k, int nF,
+                                              bool direct, int slot, int *ovf)
 {
     const int lane = threadIdx.x & 31;
-    const unsigned lt = lanemask_lt();
     const int ccap = s.ccap;
     const int i = s.fid[k];
-    const float4 qn = s.fref[k], qo = s.oref[k];
+    const float4 qn = s.fref[k];
     const int sc = flagged_scene(s, k);
     const int off = s.row_off[i], cap = s.row_cap[i], len0 = min(s.row_len[i], cap);
     const SceneGeom &g = s.sg[sc];
     // the direct test's count, loaded now (its latency under the stencil's)
-    const bool own = s.sc_cnt != nullptr;
-    const int m_dir = !direct ? 0 : own ? s.sc_cnt[slot * s.nscenes + sc] : nF;
+    const int m_dir = !direct ? 0 : s.sc_cnt ? s.sc_cnt[slot * s.nscenes + sc] : nF;
     const int d0 = g.dim[0], d1 = g.dim[1], d2 = g.dim[2];
-    const int ci = cell_key(g, qn.x, qn.y, qn.z) - g.cell_base;
-    const int cx = ci % d0, cy = (ci / d0) % d1, cz = ci / (d0 * d1);
+    const int cx = cell_coord(qn.x, g.lo[0], g.invL, d0);
+    const int cy = cell_coord(qn.y, g.lo[1], g.invL, d1);
+    const int cz = cell_coord(qn.z, g.lo[2], g.invL, d2);
     int cnt_l = 0, cid = 0;
     if (lane < 27) {
         const int x = cx + lane % 3 - 1, y = cy + (lane / 3) % 3 - 1, z = cz + lane / 9 - 1;
@@ -613,270 +673,232 @@ static __device__ __noinline__ void patch_warp(const DevState &s, int k, int nF,
             }
         }
     }
-    const int jo0 = lane < len0 ? s.col[off + lane] : -1;
+    const int tw = kDense ? tm.w : 0, per = kDense ? tm.size * 32 : 32;
+    const int e0 = tw * 32 + lane;
+    const int jo0 = e0 < len0 ? s.col[off + e0] : -2;
+    int given = 0;   // entries given out of row i (a team counts in shared memory)
+    if (kDense && tw == 0 && lane == 0) s_team_new[tm.slot] = 0;
     cnt_l = min(cnt_l, ccap);
     const int incl = warp_incl_scan(cnt_l);
     const int excl = incl - cnt_l;
     const int total = __shfl_sync(FULL, incl, 31);
-    // candidate kk of the stencil: its cell by a 5-step shuffle search
-    auto cand_idx = [&](int kk) {
-        int c = 0;
-#pragma unroll
-        for (int st = 16; st >= 1; st >>= 1)
-            c += (__shfl_sync(FULL, incl, c + st - 1) <= kk) ? st : 0;
-        const int cc = __shfl_sync(FULL, cid, c);
-        const int ex = __shfl_sync(FULL, excl, c);
-        return (long long)cc * ccap + (kk - ex);
+    if (tw == 0 && lane == 0) atomicAdd(&s_work[0], (unsigned long long)total);
+    // The stencil's candidates.  kDense: entries at .. at + 63, two to a
+    // lane, of `cell`, the first of the cells left in todo; else candidates
+    // at .. at + 31 of the run of all.
+    unsigned todo = 0u;
+    int at = 0, cnt = total, cell = 0;
+    auto next_cell = [&]() {
+        const int src = todo ? __ffs(todo) - 1 : 0;
+        cnt = todo ? __shfl_sync(FULL, cnt_l, src) : 0;
+        cell = __shfl_sync(FULL, cid, src);
+        at = 0;
     };
-    const long long idx0 = cand_idx(lane);
-    const int jc0 = lane < total ? s.cell_id[idx0] : -1;
-    const float4 rc0 = lane < total ? s.cell_ref[idx0] : make_float4(0.f, 0.f, 0.f, 0.f);
-    // 1. removals.  An old row of up to 32 entries is held in registers
-    // (jo0), so the new row may overwrite it at once: the removals of that
-    // row are only decided here and made together with the first batch of
-    // insertions (lane_edit); a longer row is done first, entry by entry.
-    int jr0 = -1;
-    for (int e0 = 0; e0 < len0; e0 += 32) {
-        const int e = e0 + lane;
-        const int j = e0 == 0 ? jo0 : (e < len0 ? s.col[off + e] : -1);
-        bool rm = false;
-        if (e < len0 && j >= 0) {
-            // the partner's flag word, reference state and radius are
-            // loaded together (one memory latency; none of them changes
-            // during the rebuild), and only an unflagged partner's pair is
-            // tested
-            const uint32_t fw = s.ubits[j >> 5];
+    if (kDense) {
+        const unsigned some = __ballot_sync(FULL, cnt_l > 0);
+        todo = __ballot_sync(FULL, cnt_l > 0 && (__popc(some & lanemask_lt()) & (tm.size - 1)) == tw);
+        next_cell();
+    }
+    // one lane's candidate(s) (R_NL -1: none, never a pair) and what finds
+    // them again: the id, or (kDense) the cell and the first one's place in it
+    struct Cand {
+        int a, b;
+        float4 r, r2;
+    };
+    auto load = [&]() {
+        Cand q{-1, at + lane, make_float4(0.f, 0.f, 0.f, -1.f), make_float4(0.f, 0.f, 0.f, -1.f)};
+        if (kDense) {
+            q.a = cell;
+            if (q.b < cnt) q.r = s.cell_ref[(long long)cell * ccap + q.b];
+            if (q.b + 32 < cnt) q.r2 = s.cell_ref[(long long)cell * ccap + q.b + 32];
+        } else {
+            int c = 0;
+#pragma unroll
+            for (int st = 16; st >= 1; st >>= 1)
+                c += (__shfl_sync(FULL, incl, c + st - 1) <= q.b) ? st : 0;
+            const int cc = __shfl_sync(FULL, cid, c);
+            const int ex = __shfl_sync(FULL, excl, c);
+            if (q.b < cnt) {
+                const long long idx = (long long)cc * ccap + (q.b - ex);
+                q.a = s.cell_id[idx];
+                q.r = s.cell_ref[idx];
+            }
+        }
+        at += kDense ? 64 : 32;
+        if (kDense && at >= cnt) {
+            todo &= todo - 1;
+            next_cell();
+        }
+        return q;
+    };
+    bool more = at < cnt;
+    Cand cand = load();
+    // the first records of the flagged list.  Many scenes: the scene's own
+    // segment of the flagged particles (scenes share one coordinate frame,
+    // so the global list would also hold far-away twins)
+    auto listed = [&](int kk, float4 &r, int &j) {
+        r = make_float4(0.f, 0.f, 0.f, 0.f);
+        j = -1;
+        if (kk < m_dir) {
+            const bool own = s.sc_cnt != nullptr;
+            r = own ? s.sfref[g.first + kk] : s.fref[kk];
+            j = own ? s.sfid[g.first + kk] : s.fid[kk];
+        }
+    };
+    float4 rf0;
+    int jf0;
+    listed(e0, rf0, jf0);
+    if (tw == 0 && lane == 0 && m_dir) atomicAdd(&s_work[1], (unsigned long long)m_dir);
+    // whether old entry j leaves row i, and (jr, at sp) whether i leaves row j:
+    // the partner's flag word, reference state, radius and row bounds are
+    // loaded together (one memory latency; none but the row's length changes
+    // during the rebuild, and that only beyond the entries it has now)
+    auto leaves = [&](int j, int &jr, RowSpan &sp) {
+        jr = -1;
+        sp = row_span(s, j);
+        if (j < 0) return false;
+        const uint32_t fw = s.ubits[j >> 5];
+        const float4 rj = s.ref[j];
+        const float rr = s.rad[j];
+        const bool fj = (fw >> (j & 31)) & 1u;
+        if (!kHist && fj) return false;
+        const bool rm = !pair_hit(qn, make_float4(rj.x, rj.y, rj.z, __fadd_rn(rr, rj.w)));
+        if (rm && !fj) jr = j;
+        return rm;
+    };
+    // 1. removals: the first entry of each lane is only decided here and its
+    // removal made together with the first insertion (lane_edit); a row
+    // longer than the team's lanes does the rest at once.
+    int jr0, edits = 0;
+    RowSpan sr0;
+    unsigned freemask = 0u;
+    {
+        const bool rm = leaves(jo0, jr0, sr0);
+        if (kHist) {
+            if (rm) s.col[off + e0] = -1;
+            freemask = __ballot_sync(FULL, jo0 == -1 || rm);
+            if (kDense && tw == 0 && lane == 0) s_team_free[tm.slot] = freemask;
+        }
+        edits += __popc(__ballot_sync(FULL, rm));
+    }
+    for (int eb = per + tw * 32; eb < len0; eb += per) {
+        const int e = eb + lane;
+        int jr;
+        RowSpan sp;
+        const bool rm = leaves(e < len0 ? s.col[off + e] : -2, jr, sp);
+        if (kHist && rm) s.col[off + e] = -1;
+        if (jr >= 0) lane_remove(s, jr, i);
+        edits += __popc(__ballot_sync(FULL, rm));
+    }
+    team_sync(tm);   // the old row has been read; the counters are set
+    if (kHist && kDense) freemask = s_team_free[tm.slot];
+    // the next entry of row i for every lane that takes one; an entry beyond
+    // the row's capacity is dropped and the row's length records the overflow
+    auto append = [&](bool take, int j) {
+        const unsigned m = __ballot_sync(FULL, take);
+        if (!m) return;
+        int a = given;
+        if (kDense) {
+            if (lane == 0) a = atomicAdd(&s_team_new[tm.slot], __popc(m));
+            a = __shfl_sync(FULL, a, 0);
+        } else {
+            given += __popc(m);
+        }
+        a += __popc(m & lanemask_lt());
+        if (take) {
+            const int nfree = __popc(freemask);
+            const int p = !kHist ? a : a < nfree ? (int)__fns(freemask, 0, a + 1) : len0 + a - nfree;
+            if (p < cap) {
+                s.col[off + p] = j;
+                if (kHist) s.hist[off + p] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
+    };
+    // the flagged partners of the direct test
+    auto flagged = [&](int j, float4 r) {
+        bool take = j >= g.first && j < g.first + g.count && j != i && pair_hit(qn, r);
+        if (kHist) take = take && !pair_hit(s.oref[k], s.pold[j]);
+        append(take, j);
+    };
+    flagged(jf0, rf0);
+    // 2. stencil and 3. insertions
+    // Candidates that pass the pair test are only noted at first (kDense: their
+    // slots, else their ids) and taken up together, up to 32 at a time: what
+    // follows from them is a chain of loads and a claim, paid once a row and
+    // not once for every cell with a partner in it (2M drum under the paper's
+    // rule: 3,500 cycles for each of the 16 cells of a row before).
+    int2 *noted = s_noted[threadIdx.x >> 5];
+    int n_noted = 0;
+    auto take_up = [&]() {
+        __syncwarp();
+        const int m = min(n_noted, 32);
+        n_noted -= m;
+        int j = -1;
+        if (lane < m) {
+            const int2 q = noted[n_noted + lane];
+            j = kDense ? s.cell_id[(long long)q.x * ccap + q.y] : q.x;
+        }
+        bool hit = j >= 0 && j != i, ins = false;   // -1: a freed slot
+        RowSpan si{0, 0, 0};
+        if (hit) {
+            si = row_span(s, j);
             const float4 rj = s.ref[j];
             const float rr = s.rad[j];
-            if (!((fw >> (j & 31)) & 1u))
-                rm = !pair_hit(qn, make_float4(rj.x, rj.y, rj.z, __fadd_rn(rr, rj.w)));
-        }
-        if (len0 <= 32) jr0 = rm ? j : -1;
-        else if (rm) lane_remove(s, j, i);
-        work[2] += __popc(__ballot_sync(FULL, rm));
-    }
-    work[0] += total;
-    // 2. stencil (+ direct test) and 3. insertions
-    int found = 0;
-    if (total == 0 && jr0 >= 0) lane_remove(s, jr0, i);
-    for (int b0 = 0; b0 < total; b0 += 32) {
-        const int kk = b0 + lane;
-        int j = -1;
-        float4 rj = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (b0 == 0) {
-            j = jc0;
-            rj = rc0;
-        } else {
-            const long long idx = cand_idx(kk);
-            if (kk < total) {
-                j = s.cell_id[idx];
-                rj = s.cell_ref[idx];
-            }
-        }
-        bool hit = false, ins = false;
-        if (kk < total && j >= 0 && j != i) {
+            const float4 qo = s.oref[k];
             const bool fj = bit_of(s.ubits, j);
-            if (!(direct && fj)) {
-                hit = pair_hit(qn, rj);
-                ins = hit && !fj && !pair_hit(qo, rj);
-            }
+            if (direct && fj) hit = false;
+            else ins = !pair_hit(qo, kHist && fj ? s.pold[j]
+                                                 : make_float4(rj.x, rj.y, rj.z, __fadd_rn(rr, rj.w)));
+            if (kHist) hit = ins;
+            ins = ins && !fj;
         }
+        append(hit, j);
+        edits += __popc(__ballot_sync(FULL, ins));
+        lane_edit(s, jr0, sr0, ins ? j : -1, si, i, ovf);
+        jr0 = -1;
+        __syncwarp();
+    };
+    auto note = [&](float4 r, int a, int b) {
+        const bool hit = r.w >= 0.0f && pair_hit(qn, r);
         const unsigned m = __ballot_sync(FULL, hit);
-        if (hit) {
-            const int p = found + __popc(m & lt);
-            if (p < cap) s.col[off + p] = j;
-        }
-        found += __popc(m);
-        work[2] += __popc(__ballot_sync(FULL, ins));
-        if (b0 == 0) {
-            lane_edit(s, jr0, ins ? j : -1, i, ovf);
-        } else if (ins) {
-            lane_insert(s, j, i, ovf);
-        }
+        if (!m) return;
+        if (n_noted + __popc(m) > kNoted) take_up();
+        if (hit) noted[n_noted + __popc(m & lanemask_lt())] = make_int2(a, b);
+        n_noted += __popc(m);
+    };
+    while (more) {   // the next candidates in flight while these are tested
+        more = at < cnt;
+        const Cand next = load();
+        note(cand.r, cand.a, cand.b);
+        if (kDense) note(cand.r2, cand.a, cand.b + 32);
+        cand = next;
     }
-    if (direct) {
-        // kDirectUnroll reference states and ids per lane in flight (one
-        // memory latency a batch).  Many scenes: the scene's own segment of
-        // the flagged particles (scenes share one coordinate frame, so the
-        // global list would also hold far-away twins)
-        const float4 *lst = own ? s.sfref + g.first : s.fref;
-        const int *ids = own ? s.sfid + g.first : s.fid;
-        const int m = m_dir;
-        work[1] += m;
-        for (int b0 = 0; b0 < m; b0 += 32 * kDirectUnroll) {
-            float4 rf[kDirectUnroll];
-            int jf[kDirectUnroll];
+    do take_up();   // (once in any case: the removals of the old row)
+    while (n_noted > 0);
+    // the rest of the flagged list, kDirectUnroll records per lane in flight
+    for (int b0 = per + tw * 32 * kDirectUnroll; b0 < m_dir; b0 += per * kDirectUnroll) {
+        float4 rf[kDirectUnroll];
+        int jf[kDirectUnroll];
 #pragma unroll
-            for (int u = 0; u < kDirectUnroll; ++u) {
-                const int kk = b0 + u * 32 + lane;
-                rf[u] = kk < m ? lst[kk] : make_float4(0.f, 0.f, 0.f, 0.f);
-                jf[u] = kk < m ? ids[kk] : -1;
-            }
-#pragma unroll
-            for (int u = 0; u < kDirectUnroll; ++u) {
-                const int kk = b0 + u * 32 + lane;
-                int j = -1;
-                if (kk < m && pair_hit(qn, rf[u])) {
-                    j = jf[u];
-                    if (j == i || j < g.first || j >= g.first + g.count) j = -1;
-                }
-                const unsigned msk = __ballot_sync(FULL, j >= 0);
-                if (j >= 0) {
-                    const int p = found + __popc(msk & lt);
-                    if (p < cap) s.col[off + p] = j;
-                }
-                found += __popc(msk);
-            }
+        for (int u = 0; u < kDirectUnroll; ++u) {
+            listed(b0 + u * 32 + lane, rf[u], jf[u]);
         }
+#pragma unroll
+        for (int u = 0; u < kDirectUnroll; ++u) flagged(jf[u], rf[u]);
     }
-    for (int e = found + lane; e < len0; e += 32) s.col[off + e] = -1;
+    if (lane == 0 && edits) atomicAdd(&s_work[2], (unsigned long long)edits);
+    team_sync(tm);
+    if (tw != 0) return;
+    if (kDense) {
+        given = s_team_new[tm.slot];
+        __syncwarp();   // read by every lane before the next patch clears it
+    }
+    const int len = !kHist ? given : len0 + max(given - __popc(freemask), 0);
+    if (!kHist)
+        for (int e = given + lane; e < len0; e += 32) s.col[off + e] = -1;
     if (lane == 0) {
-        s.row_len[i] = found;
-        if (found > cap) atomicExch(ovf, 1);
-    }
-}
-
-// The reference record (xref, R_NL) of particle j as it was before this
-// step's updates: its old record if it was updated at this step (history
-// mode keeps it in pold), else its present one.
-__device__ __forceinline__ float4 old_record(const DevState &s, int j)
-{
-    if (bit_of(s.ubits, j)) return s.pold[j];
-    const float4 r = s.ref[j];
-    return make_float4(r.x, r.y, r.z, __fadd_rn(s.rad[j], r.w));
-}
-
-// Appends the partners j of the lanes with `ins` to row i, which only this
-// warp edits: first into the row's free slots among its first 32 entries
-// (bits of *freemask), then at its end (*tail); each new entry's history
-// starts at zero.  An entry past the row's capacity is dropped and the
-// row's length records the overflow (the re-layout rebuilds the row).
-__device__ __forceinline__ void own_row_insert(const DevState &s, int off, int cap, bool ins,
-                                               int j, unsigned *freemask, int *tail)
-{
-    const unsigned m = __ballot_sync(FULL, ins);
-    if (!m) return;
-    const int cnt = __popc(m), nfree = __popc(*freemask);
-    const int rank = __popc(m & lanemask_lt());
-    if (ins) {
-        const int slot = rank < nfree ? (int)__fns(*freemask, 0, rank + 1) : *tail + rank - nfree;
-        if (slot < cap) {
-            s.col[off + slot] = j;
-            s.hist[off + slot] = make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
-    const int used = min(cnt, nfree);
-    for (int t = 0; t < used; ++t) *freemask &= *freemask - 1;   // lowest bits taken
-    *tail += cnt - used;
-}
-
-// a4 + a5 for flagged particle k with contact history (LVB_OPT_HISTORY):
-// the same pair decisions as patch_warp, but row i is edited in place, as
-// the unflagged rows are, so that a partner that stays a pair keeps its
-// slot -- and its history -- through the rebuild:
-//   1. each old entry j no longer a pair under the new reference states of
-//      i and j (this step's updates are all written) becomes -1, and i
-//      leaves row j if j is unflagged (a flagged j edits its own row);
-//   2. each partner found by the stencil (+ the direct flagged test) that
-//      is a pair now and was not one under the old states (the old record
-//      of a flagged partner is kept in pold) joins row i with zero
-//      history, and an unflagged partner gets i in its row.
-static __device__ __noinline__ void patch_warp_hist(const DevState &s, int k, int nF, bool direct,
-                                                    int slot, int *ovf, unsigned (&work)[3])
-{
-    const int lane = threadIdx.x & 31;
-    const int ccap = s.ccap;
-    const int i = s.fid[k];
-    const float4 qn = s.fref[k], qo = s.oref[k];
-    const int sc = flagged_scene(s, k);
-    const int off = s.row_off[i], cap = s.row_cap[i], len0 = min(s.row_len[i], cap);
-    const SceneGeom &g = s.sg[sc];
-    const int d0 = g.dim[0], d1 = g.dim[1], d2 = g.dim[2];
-    const int ci = cell_key(g, qn.x, qn.y, qn.z) - g.cell_base;
-    const int cx = ci % d0, cy = (ci / d0) % d1, cz = ci / (d0 * d1);
-    int cnt_l = 0, cid = 0;
-    if (lane < 27) {
-        const int x = cx + lane % 3 - 1, y = cy + (lane / 3) % 3 - 1, z = cz + lane / 9 - 1;
-        if (x >= 0 && x < d0 && y >= 0 && y < d1 && z >= 0 && z < d2) {
-            const float dd = s.reach ? cell_dist2(g, x, y, z, qn) : 0.0f;
-            if (s.reach == 0 || within_reach(g, dd, qn.w, g.H)) {
-                cid = g.cell_base + (z * d1 + y) * d0 + x;
-                cnt_l = s.cell_cnt[cid];
-                if (s.reach == 2 && !within_reach(g, dd, qn.w, __int_as_float(s.cell_rmax[cid])))
-                    cnt_l = 0;
-            }
-        }
-    }
-    cnt_l = min(cnt_l, ccap);
-    const int incl = warp_incl_scan(cnt_l);
-    const int excl = incl - cnt_l;
-    const int total = __shfl_sync(FULL, incl, 31);
-    work[0] += total;
-    // 1. old entries
-    unsigned freemask = 0u;
-    for (int e0 = 0; e0 < len0; e0 += 32) {
-        const int e = e0 + lane;
-        const int j = e < len0 ? s.col[off + e] : -2;
-        bool rm = false;
-        if (j >= 0) {
-            const float4 rj = s.ref[j];
-            rm = !pair_hit(qn, make_float4(rj.x, rj.y, rj.z, __fadd_rn(s.rad[j], rj.w)));
-            if (rm) {
-                s.col[off + e] = -1;
-                if (!bit_of(s.ubits, j)) lane_remove(s, j, i);
-            }
-        }
-        const unsigned fm = __ballot_sync(FULL, e < len0 && (j == -1 || rm));
-        if (e0 == 0) freemask = fm;
-        work[2] += __popc(__ballot_sync(FULL, rm));
-    }
-    int tail = len0;
-    // 2. stencil
-    for (int b0 = 0; b0 < total; b0 += 32) {
-        const int kk = b0 + lane;
-        int c = 0;
-#pragma unroll
-        for (int st = 16; st >= 1; st >>= 1)
-            c += (__shfl_sync(FULL, incl, c + st - 1) <= kk) ? st : 0;
-        const int cc = __shfl_sync(FULL, cid, c);
-        const int ex = __shfl_sync(FULL, excl, c);
-        int j = -1;
-        float4 rj = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (kk < total) {
-            const long long idx = (long long)cc * ccap + (kk - ex);
-            j = s.cell_id[idx];
-            rj = s.cell_ref[idx];
-        }
-        bool ins = false, fj = false;
-        if (kk < total && j >= 0 && j != i) {
-            fj = bit_of(s.ubits, j);
-            if (!(direct && fj) && pair_hit(qn, rj))
-                ins = !pair_hit(qo, fj ? s.pold[j] : rj);
-        }
-        own_row_insert(s, off, cap, ins, j, &freemask, &tail);
-        work[2] += __popc(__ballot_sync(FULL, ins && !fj));
-        if (ins && !fj) lane_insert(s, j, i, ovf);
-    }
-    if (direct) {
-        const bool own = s.sc_cnt != nullptr;
-        const float4 *lst = own ? s.sfref + g.first : s.fref;
-        const int *ids = own ? s.sfid + g.first : s.fid;
-        const int m = own ? s.sc_cnt[slot * s.nscenes + sc] : nF;
-        work[1] += m;
-        for (int b0 = 0; b0 < m; b0 += 32) {
-            const int kk = b0 + lane;
-            int j = -1;
-            if (kk < m && pair_hit(qn, lst[kk])) {
-                j = ids[kk];
-                if (j == i || j < g.first || j >= g.first + g.count) j = -1;
-            }
-            const bool ins = j >= 0 && !pair_hit(qo, s.pold[j]);
-            own_row_insert(s, off, cap, ins, j, &freemask, &tail);
-        }
-    }
-    if (lane == 0) {
-        s.row_len[i] = tail;
-        if (tail > cap) atomicExch(ovf, 1);
+        s.row_len[i] = len;
+        if (len > cap) atomicExch(ovf, 1);
     }
 }
 
@@ -997,10 +1019,6 @@ __device__ __forceinline__ unsigned long long ld_acquire(const unsigned long lon
 // the barrier state of this block (used by its thread 0 only)
 static __shared__ unsigned long long s_bar_need;   // arrivals up to the last barrier
 static __shared__ int s_bar_slot;                  // slot of the step
-// the block's share of the partial rebuilds' work counts (DevCounters
-// alg_*), gathered by its warps with shared-memory atomics and added to the
-// context's counters by thread 0 once per kernel
-static __shared__ unsigned long long s_work[3];
 // the block's rebuild work items when traced: first start, last end,
 // longest item (item_start / item_stop)
 static __shared__ unsigned long long s_items[3];
@@ -1666,51 +1684,74 @@ __device__ __forceinline__ void items_flush(const DevState &s)
     }
 }
 
-// The rebuild of a partial step (nF flagged).  Up to s.direct_max
-// flagged particles: moves and patches in one phase, on different warps
-// (work items 0..nF-1 patch rows, nF..2nF-1 move cell slots; the patches
-// skip the flagged particles in the cells and test them directly); more:
-// the moves first and a barrier, then the patches on final cells.  Returns
-// false when the step must be abandoned.
-static __device__ __noinline__ bool partial_pass(const DevState &s, int nF, int slot, int *ovf)
+constexpr int kTeamSlots = 64;   // slots per cell above which rows are patched by teams
+
+// The patches of a partial step: patch k by team k, teams round the blocks
+// first (so that a few flagged particles spread over all SMs instead of
+// filling the first blocks).  More patches than teams (which are single warps
+// then): each warp that is done takes the next one, asked for when it began
+// (the longest patch costs three times the mean).
+template <bool kHist, bool kDense>
+static __device__ __noinline__ void patch_pass(const DevState &s, int nF, bool direct, int slot,
+                                               int lg, int *ovf)
 {
-    // work items go round the blocks first (item w to block w % grid), so
-    // that a few flagged particles spread over all SMs instead of filling
-    // the warps of the first blocks
-    const int w0 = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    const bool direct = nF <= s.direct_max;
-    unsigned work[3] = {0u, 0u, 0u};
+    const int warp = threadIdx.x >> 5;
+    const Team tm{1 << lg, warp & ((1 << lg) - 1), warp >> lg};
+    const int teams = (int)(gridDim.x * (blockDim.x >> 5)) >> lg;
+    for (int k = tm.slot * (int)gridDim.x + (int)blockIdx.x; k < nF;) {
+        int next = 0;
+        if (nF > teams && (threadIdx.x & 31) == 0) next = atomicAdd(&s.cnt->next_patch[slot], 1);
+        item_start(s);
+        patch_row<kHist, kDense>(s, tm, k, nF, direct, slot, ovf);
+        item_stop(s);
+        if (nF <= teams) break;
+        k = teams + __shfl_sync(FULL, next, 0);
+    }
+}
+
+// The moves of a partial step: move k by the k-th warp from the end, in the
+// same order.
+static __device__ __noinline__ void move_pass(const DevState &s, int nF)
+{
+    const int nw = (int)(gridDim.x * (blockDim.x >> 5));
+    for (int k = nw - 1 - (int)((threadIdx.x >> 5) * gridDim.x + blockIdx.x); k < nF; k += nw) {
+        item_start(s);
+        move_warp(s, s.fid[k], s.fref[k], flagged_scene(s, k));
+        item_stop(s);
+    }
+}
+
+// The rebuild of a partial step (nF flagged).  Up to s.direct_max
+// flagged particles: moves and patches in one phase, on different warps (the
+// patches skip the flagged particles in the cells and test them directly);
+// more: the moves first and a barrier, then the patches on final cells.
+// In dense cells (more than kTeamSlots slots) a team has as many warps (1, 4,
+// 8, 16 or 32) as leave every patch a team and every move a warp of its own
+// (1M drum with friction, 930 flagged: rebuild 41 us with single warps, 25 us
+// with teams of four, before the candidates were noted).  In sparse cells a
+// row has some 20 candidates, which one warp loads at once, and the team's
+// barriers only add to its chain (settling 200k: 23.8 -> 25.3 us a step).
+// Returns false when the step must be abandoned.
+__device__ __forceinline__ bool partial_pass(const DevState &s, int nF, int slot, int *ovf)
+{
+    const int wpb = blockDim.x >> 5, nw = gridDim.x * wpb;
+    const bool direct = nF <= s.direct_max, dense = s.ccap > kTeamSlots;
+    int lg = 0;   // log2 of the team's size
+    if (dense && nF <= nw)   // (no product beyond 32 bits)
+        for (int t = 2; t <= 5; ++t)
+            if ((1 << t) <= wpb && nF * ((1 << t) + (direct ? 1 : 0)) <= nw) lg = t;
     if (!direct) {
-        for (int k = w0; k < nF; k += nw) {
-            item_start(s);
-            move_warp(s, s.fid[k], s.fref[k], flagged_scene(s, k));
-            item_stop(s);
-        }
+        move_pass(s, nF);
         if (!grid_barrier(s)) return false;
-        for (int k = w0; k < nF; k += nw) {
-            item_start(s);
-            if (s.hist) patch_warp_hist(s, k, nF, false, slot, ovf, work);
-            else patch_warp(s, k, nF, false, slot, ovf, work);
-            item_stop(s);
-        }
+    }
+    if (dense) {
+        if (s.hist) patch_pass<true, true>(s, nF, direct, slot, lg, ovf);
+        else patch_pass<false, true>(s, nF, direct, slot, lg, ovf);
     } else {
-        for (int w = w0; w < 2 * nF; w += nw) {
-            item_start(s);
-            if (w < nF) {
-                if (s.hist) patch_warp_hist(s, w, nF, true, slot, ovf, work);
-                else patch_warp(s, w, nF, true, slot, ovf, work);
-            } else {
-                move_warp(s, s.fid[w - nF], s.fref[w - nF], flagged_scene(s, w - nF));
-            }
-            item_stop(s);
-        }
+        if (s.hist) patch_pass<true, false>(s, nF, direct, slot, lg, ovf);
+        else patch_pass<false, false>(s, nF, direct, slot, lg, ovf);
     }
-    if ((threadIdx.x & 31) == 0) {
-#pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (work[q]) atomicAdd(&s_work[q], (unsigned long long)work[q]);
-    }
+    if (direct) move_pass(s, nF);
     return true;
 }
 
@@ -1772,6 +1813,7 @@ __device__ __forceinline__ bool finish_step(const DevState &s, const lvb_mlp_wei
         // stores and reductions only: no load on the step's last path
         c->nF_acc[spent] = 0;
         c->nE_acc[spent] = 0;
+        c->next_patch[spent] = 0;
         c->ovf[spent] = 0;
         c->nF = nV;
         if (s.nf_out) *s.nf_out = nV;
