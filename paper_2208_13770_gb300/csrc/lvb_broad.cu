@@ -168,8 +168,10 @@ k_rows(DevState s, int gate, int fill, int carry = 0)
     if (!nitems) return;
     count_kernel(s);
     tr_enter(s, TR_ROWS);
-    ph_rows(s, nitems, fill, (blockIdx.x * kThreads + threadIdx.x) >> 5,
-            (gridDim.x * kThreads) >> 5, &s.cnt->row_overflow, carry != 0);
+    const int w0 = (blockIdx.x * kThreads + threadIdx.x) >> 5, nw = (gridDim.x * kThreads) >> 5;
+    if (s.ccap > kTeamSlots)
+        ph_rows_dense(s, fill, w0, nw, &s.cnt->row_overflow, carry != 0);
+    else ph_rows(s, nitems, fill, w0, nw, &s.cnt->row_overflow, carry != 0);
     tr_exit(s, TR_ROWS);
 }
 
@@ -604,7 +606,7 @@ int size_step(lvb_ctx *c)
     int dev = 0, sms = 0, per_sm = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int smem = check_smem_bytes(c->block_threads);
+    const int smem = c->s.check_regs ? 0 : check_smem_bytes(c->block_threads);
     // the attribute belongs to the kernel, for every context of the process:
     // always the largest any block size needs
     if (e == cudaSuccess)
@@ -1246,7 +1248,14 @@ int lvb_set_option(lvb_ctx *c, int32_t option, int64_t value)
         s.early_beta = (float)((double)value / 1000.0);
     } else if (option == LVB_OPT_CHECK_LOADS) {
         if (value != LVB_CHECK_REGS && value != LVB_CHECK_RING) return LVB_EINVAL;
+        const int old = c->s.check_regs;
         c->s.check_regs = value == LVB_CHECK_REGS;
+        const int rc = size_step(c);   // the ring's shared memory counts
+        if (rc) {
+            c->s.check_regs = old;
+            size_step(c);
+            return rc;
+        }
     } else if (option == LVB_OPT_STENCIL_REACH) {
         if (value < 0 || value > 2) return LVB_EINVAL;
         c->s.reach = (int)value;

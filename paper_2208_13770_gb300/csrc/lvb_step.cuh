@@ -595,8 +595,10 @@ __device__ __forceinline__ void team_sync(const Team &t)
 // context's counters by thread 0 once per kernel
 static __shared__ unsigned long long s_work[3];
 
+constexpr int kTeamSlots = 64;   // slots per cell above which cells count as dense
+
 constexpr int kNoted = 64;   // candidates a warp notes before it takes them up
-static __shared__ int2 s_noted[kStepMaxThreads / 32][kNoted];
+static __shared__ __align__(16) int2 s_noted[kStepMaxThreads / 32][kNoted];
 static __shared__ int s_team_new[kStepMaxThreads / 32];       // entries given out of the row
 static __shared__ unsigned s_team_free[kStepMaxThreads / 32]; // its free slots (history)
 
@@ -986,6 +988,127 @@ __device__ __forceinline__ void ph_rows(const DevState &s, int nitems, int fill,
         if (lane == 0) {
             s.row_len[i] = found;
             if (fill && found > cap) atomicExch(ovf, 1);
+        }
+    }
+}
+
+// The same in dense cells (more than kTeamSlots slots): a warp takes 32 slots
+// of a cell at a time, one row to a lane, and each of the 27 cells around it in
+// turn.  One ballot tells which of the rows reach that cell at all; its
+// candidates are held 32 at a time, one to a lane, and every such row is
+// tested against them from shared memory.  What bounds it is instruction
+// issue, the tests themselves: a test of 32 candidates is a broadcast and
+// the formula, with no load, address or search of its own (1M lognormal drum,
+// 230 candidates a row for 6 partners, the whole list at every step: 1,421 us
+// with a warp to a row and a flattened run of its candidates, 1,360 with a
+// warp to a row and its cells one after another at 925 instructions a row,
+// 899 this way at 590; two or four rows tested together: 928 and 960).
+// Warps w0, w0 + wstride, ... take the cells round and round, the next 32 slots
+// of the same cell by another warp.
+__device__ __forceinline__ void ph_rows_dense(const DevState &s, int fill, int w0, int wstride,
+                                              int *ovf, bool carry)
+{
+    const int lane = threadIdx.x & 31;
+    const int ccap = s.ccap;
+    float4 *rows = reinterpret_cast<float4 *>(s_noted[threadIdx.x >> 5]);
+    static_assert(kNoted * sizeof(int2) >= 32 * sizeof(float4), "the rows' records fit");
+    for (int e0 = 0; e0 < ccap; e0 += 32) {
+        const int first = (int)(((long long)w0 + 61LL * (e0 >> 5)) % wstride);
+        for (long long k0 = first; k0 < s.ncells; k0 += 32LL * wstride) {
+            const long long mine = k0 + (long long)lane * wstride;
+            const int filled = mine < s.ncells ? min(s.cell_cnt[mine], ccap) : 0;
+            for (unsigned left = __ballot_sync(FULL, filled > e0); left; left &= left - 1) {
+                const int src = __ffs(left) - 1;
+                const int cell = (int)(k0 + (long long)src * wstride);
+                const int e = e0 + lane;
+                // lane l: one row of this cell
+                int id = -1, off = 0, cap = 0, found = 0;
+                float4 q = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (e < __shfl_sync(FULL, filled, src)) {
+                    id = s.cell_id[(long long)cell * ccap + e];   // -1: a freed slot
+                    q = s.cell_ref[(long long)cell * ccap + e];
+                }
+                const unsigned valid = __ballot_sync(FULL, id >= 0);
+                if (!valid) continue;
+                if (fill && id >= 0) {
+                    off = s.row_off[id];
+                    cap = s.row_cap[id];
+                }
+                __syncwarp();
+                rows[lane] = q;
+                __syncwarp();
+                const SceneGeom &g = geom_of(s, __shfl_sync(FULL, id, __ffs(valid) - 1));
+                // lane l < 27: a cell around this one, its filled slots and bound
+                const int d0 = g.dim[0], d1 = g.dim[1], d2 = g.dim[2], ci = cell - g.cell_base;
+                const int cx = ci % d0, cy = (ci / d0) % d1, cz = ci / (d0 * d1);
+                int near = 0, cnt_l = 0;
+                float bound_l = g.H;
+                {
+                    const int x = cx + lane % 3 - 1, y = cy + (lane / 3) % 3 - 1, z = cz + lane / 9 - 1;
+                    if (lane < 27 && x >= 0 && x < d0 && y >= 0 && y < d1 && z >= 0 && z < d2) {
+                        near = g.cell_base + (z * d1 + y) * d0 + x;
+                        cnt_l = min(s.cell_cnt[near], ccap);
+                        if (s.reach == 2)
+                            bound_l = fminf(bound_l, __int_as_float(s.cell_rmax[near]));
+                    }
+                }
+                for (unsigned cells = __ballot_sync(FULL, cnt_l > 0); cells; cells &= cells - 1) {
+                    const int t = __ffs(cells) - 1;
+                    const long long at = (long long)__shfl_sync(FULL, near, t) * ccap + lane;
+                    const int cnt = __shfl_sync(FULL, cnt_l, t);
+                    const float bound = __shfl_sync(FULL, bound_l, t);
+                    const unsigned reach = __ballot_sync(
+                        FULL, id >= 0 && (s.reach == 0 ||
+                                          within_reach(g,
+                                                       cell_dist2(g, cx + t % 3 - 1,
+                                                                  cy + (t / 3) % 3 - 1,
+                                                                  cz + t / 9 - 1, q),
+                                                       q.w, bound)));
+                    if (!reach) continue;
+                    for (int c0 = 0; c0 < cnt; c0 += 32) {
+                        // lane l: candidate c0 + l of that cell (none: infinitely far)
+                        int j = -1;
+                        float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (c0 + lane < cnt) {
+                            j = s.cell_id[at + c0];
+                            r = s.cell_ref[at + c0];
+                        }
+                        if (j < 0) r.x = INFINITY;
+                        for (unsigned todo = reach; todo; todo &= todo - 1) {
+                            const int p = __ffs(todo) - 1;
+                            const bool close = pair_hit(rows[p], r);
+                            if (!__any_sync(FULL, close)) continue;
+                            const int i = __shfl_sync(FULL, id, p);
+                            const bool hit = close && j != i;
+                            const unsigned m = __ballot_sync(FULL, hit);
+                            if (fill) {
+                                const int ro = __shfl_sync(FULL, off, p);
+                                const int rc = __shfl_sync(FULL, cap, p);
+                                const int o =
+                                    __shfl_sync(FULL, found, p) + __popc(m & lanemask_lt());
+                                if (hit && o < rc) {
+                                    s.col[ro + o] = j;
+                                    if (s.hist)
+                                        s.hist[ro + o] = carry ? carried_history(s, i, j)
+                                                               : make_float4(0.f, 0.f, 0.f, 0.f);
+                                }
+                            }
+                            if (lane == p) found += __popc(m);
+                        }
+                    }
+                }
+                if (id >= 0) {
+                    s.row_len[id] = found;
+                    if (fill && found > cap) atomicExch(ovf, 1);
+                }
+                if (fill)
+                    for (unsigned todo = valid; todo; todo &= todo - 1) {
+                        const int p = __ffs(todo) - 1;
+                        const int ro = __shfl_sync(FULL, off, p), rc = __shfl_sync(FULL, cap, p);
+                        for (int o = __shfl_sync(FULL, found, p) + lane; o < rc; o += 32)
+                            s.col[ro + o] = -1;
+                    }
+            }
         }
     }
 }
@@ -1439,7 +1562,8 @@ static __device__ __noinline__ void all_rows_pass(const DevState &s, int fill, i
                                                   bool carry = false)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    ph_rows(s, s.n, fill, t >> 5, nt >> 5, ovf, carry);
+    if (s.ccap > kTeamSlots) ph_rows_dense(s, fill, t >> 5, nt >> 5, ovf, carry);
+    else ph_rows(s, s.n, fill, t >> 5, nt >> 5, ovf, carry);
 }
 
 // Contact history: the rows as they stand (offsets, lengths, entries and
@@ -1683,8 +1807,6 @@ __device__ __forceinline__ void items_flush(const DevState &s)
         s_items[1] = s_items[2] = 0ULL;
     }
 }
-
-constexpr int kTeamSlots = 64;   // slots per cell above which rows are patched by teams
 
 // The patches of a partial step: patch k by team k, teams round the blocks
 // first (so that a few flagged particles spread over all SMs instead of

@@ -72,3 +72,31 @@ def test_teams_match_the_oracle(orc, moved, history, threads):
     assert st["cell_capacity"] >= 512
     assert np.diff(rows).max() > 32
     ctx.close()
+
+
+@pytest.mark.parametrize("trigger", [1, 2])
+@pytest.mark.parametrize("reach", [0, 1, 2])
+@pytest.mark.parametrize("n", [1, 33, 6000])
+def test_whole_lists_match_the_oracle(orc, trigger, reach, n):
+    # every row built anew, a lane to a row (cells of 1 to some 100 spheres)
+    lvb = _lvb()
+    from oracle.statemachine import OracleLVB
+    s, _ = _bed(n, 23)
+    pos = s.pos.astype(np.float32)
+    ctx = lvb.LVB(torch.from_numpy(pos).cuda(), s.lo, s.hi, lvb.LVB_SKIN_DIAMETER_FACTOR, 0.1,
+                  s.dt, trigger, 1.25)
+    ctx.set_option(lvb.LVB_OPT_CELL_CAPACITY, 200)
+    ctx.set_option(lvb.LVB_OPT_STENCIL_REACH, reach)
+    sm = OracleLVB(pos, orc.SKIN_DIAMETER_FACTOR, 0.1, s.dt, ctx.stats()["rnl_max"], trigger)
+    rng = np.random.default_rng(n)
+    x = pos.copy()
+    for _ in range(3):
+        x[:, :3] += rng.normal(0.0, 2e-4, size=(n, 3)).astype(np.float32)
+        ctx.step(torch.from_numpy(x).cuda())
+        sm.step(x)
+        pi, pj = ctx.pairs_ij()
+        assert np.array_equal(pi, sm.pi) and np.array_equal(pj, sm.pj)
+        rows, col = ctx.pairs_csr()
+        assert rows[-1] == 2 * len(pi) == len(col)
+    assert ctx.stats()["cell_capacity"] >= 200
+    ctx.close()
