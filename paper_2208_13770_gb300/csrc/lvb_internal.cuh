@@ -56,6 +56,7 @@ struct DevCounters {
     long long store_needed;  // entries the row store needed at the last layout
     unsigned long long kernels;  // kernels of this library executed (device count)
     unsigned long long barriers; // grid barriers passed by step kernels
+    long long ex_total;      // entries of the last export
     long long log_n;         // rebuild-log samples closed so far
     // work of the partial rebuilds so far (for the algorithmic byte count):
     // stencil candidates read, flagged-list records read by the direct
