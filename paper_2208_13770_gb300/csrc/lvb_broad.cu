@@ -975,16 +975,6 @@ int export_scan(lvb_ctx *c, long long *total)
     return LVB_OK;
 }
 
-bool on_device(const void *p)
-{
-    cudaPointerAttributes a{};
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();   // an unknown pointer: host memory
-        return false;
-    }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
-}
-
 int copy_out(lvb_ctx *c, void *dst, const void *src, size_t bytes)
 {
     if (!bytes) return LVB_OK;
@@ -1809,10 +1799,20 @@ cudaStream_t step_stream(lvb_ctx *c)
     return c->stream;
 }
 
-void small_scratch(lvb_ctx *c, unsigned **u32, unsigned long long **u64)
+int sync_counters_of(lvb_ctx *c, const DevCounters **host)
 {
-    *u32 = c->scratch;
-    *u64 = c->sum64;
+    *host = c->cnt_h;
+    return sync_counters(c);
+}
+
+bool on_device(const void *p)
+{
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();   // an unknown pointer: host memory
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
 }
 
 int grow_stores_if_asked(lvb_ctx *c)

@@ -57,6 +57,8 @@ struct DevCounters {
     unsigned long long kernels;  // kernels of this library executed (device count)
     unsigned long long barriers; // grid barriers passed by step kernels
     long long ex_total;      // entries of the last export
+    unsigned long long clump_total;   // sub-sphere contacts of the last clump call
+    unsigned clump_bad;      // and what was wrong with its inputs (CL_BAD_*)
     long long log_n;         // rebuild-log samples closed so far
     // work of the partial rebuilds so far (for the algorithmic byte count):
     // stencil candidates read, flagged-list records read by the direct
@@ -321,9 +323,11 @@ RowsView rows_view(lvb_ctx *c);
 DevState step_state(lvb_ctx *c);
 void step_shape(lvb_ctx *c, int *blocks, int *threads);
 cudaStream_t step_stream(lvb_ctx *c);
-// The context's small device scratch (at least 8 words and one 64-bit
-// word), used on its stream by calls that synchronise before returning.
-void small_scratch(lvb_ctx *c, unsigned **u32, unsigned long long **u64);
+// Waits for the context's stream and reads its counters back: the sticky device
+// error, and the counters through *host (valid until the next such call).
+int sync_counters_of(lvb_ctx *c, const DevCounters **host);
+// Whether p is memory that kernels may write in place (device or managed).
+bool on_device(const void *p);
 
 // Changes whenever the step kernel's arguments or launch shape change
 // (options, logging, store growth), so that a caller that keeps a launch
