@@ -741,7 +741,7 @@ void free_all(lvb_ctx *c)
                     c->scratch, c->sum64, c->sg_d, c->scene_of_d, s.born, s.cell_live,
                     s.cell_rmax,
                     s.lg_feat, s.lg_x, s.lg_t, s.lg_m, s.log_buf,
-                    s.hist, s.pold, s.old_off, s.old_len, s.old_col, s.old_hist};
+                    s.hist, s.live, s.pold, s.old_off, s.old_len, s.old_col, s.old_hist};
     for (void *p : ptrs)
         if (p) cudaFree(p);
     if (c->cnt_h) cudaFreeHost(c->cnt_h);
@@ -1532,14 +1532,16 @@ int lvb_set_option(lvb_ctx *c, int32_t option, int64_t value)
         const cudaError_t ee = cudaStreamSynchronize(c->stream);
         if (ee != cudaSuccess) return from_cuda(ee);
         DevState &s = c->s;
-        void *ptrs[] = {s.hist, s.pold, s.old_off, s.old_len, s.old_col, s.old_hist};
+        void *ptrs[] = {s.hist, s.live, s.pold, s.old_off, s.old_len, s.old_col, s.old_hist};
         for (void *q : ptrs)
             if (q) cudaFree(q);
         s.hist = s.pold = s.old_hist = nullptr;
+        s.live = nullptr;
         s.old_off = s.old_len = s.old_col = nullptr;
         c->history = false;
         if (value) {
             cudaError_t e = dalloc(&s.hist, c->col_alloc);
+            if (e == cudaSuccess) e = dalloc(&s.live, c->n);
             if (e == cudaSuccess) e = dalloc(&s.pold, c->n);
             if (e == cudaSuccess) e = dalloc(&s.old_off, c->n);
             if (e == cudaSuccess) e = dalloc(&s.old_len, c->n);
@@ -1547,12 +1549,15 @@ int lvb_set_option(lvb_ctx *c, int32_t option, int64_t value)
             if (e == cudaSuccess) e = dalloc(&s.old_hist, c->col_alloc);
             if (e == cudaSuccess)
                 e = cudaMemsetAsync(s.hist, 0, sizeof(float4) * (size_t)c->col_alloc, c->stream);
+            if (e == cudaSuccess)
+                e = cudaMemsetAsync(s.live, 0, sizeof(unsigned) * (size_t)c->n, c->stream);
             if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
             if (e != cudaSuccess) {
-                void *qs[] = {s.hist, s.pold, s.old_off, s.old_len, s.old_col, s.old_hist};
+                void *qs[] = {s.hist, s.live, s.pold, s.old_off, s.old_len, s.old_col, s.old_hist};
                 for (void *q : qs)
                     if (q) cudaFree(q);
                 s.hist = s.pold = s.old_hist = nullptr;
+                s.live = nullptr;
                 s.old_off = s.old_len = s.old_col = nullptr;
                 return from_cuda(e);
             }
@@ -1772,6 +1777,7 @@ RowsView rows_view(lvb_ctx *c)
     v.row_cap = c->s.row_cap;
     v.col = c->s.col;
     v.hist = c->s.hist;
+    v.live = c->s.live;
     v.rad = c->s.rad;
     v.kernels = &c->s.cnt->kernels;
     v.cnt = c->s.cnt;

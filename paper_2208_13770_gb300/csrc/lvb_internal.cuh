@@ -307,6 +307,8 @@ struct RowsView {
     const int *row_cap;
     const int *col;
     float4 *hist;                  // contact history beside col, or null
+    unsigned *live;                // per particle, which of its row's first 32 records
+                                   // may be other than zero (null without history)
     const float *rad;
     unsigned long long *kernels;   // device kernel counter of the context
     DevCounters *cnt;              // counters (trace slots)

@@ -118,6 +118,9 @@ struct DevState {
     // beside col[e], kept with its entry through partial rebuilds,
     // re-layouts and store growth; null when off
     float4 *hist;
+    unsigned *live;   // per particle, a bit for each of its row's first 32
+                      // entries whose record may be other than zero (kept by
+                      // the forces; all set when the row is laid out anew)
     float4 *pold;     // per particle: the old (xref, R_NL) of a particle
                       // updated at this step (written by its update)
     // the rows as they were before a re-layout, for carrying history
@@ -987,6 +990,7 @@ __device__ __forceinline__ void ph_rows(const DevState &s, int nitems, int fill,
             for (int e = found + lane; e < cap; e += 32) s.col[off + e] = -1;
         if (lane == 0) {
             s.row_len[i] = found;
+            if (fill && s.hist) s.live[i] = ~0u;
             if (fill && found > cap) atomicExch(ovf, 1);
         }
     }
@@ -1099,6 +1103,7 @@ __device__ __forceinline__ void ph_rows_dense(const DevState &s, int fill, int w
                 }
                 if (id >= 0) {
                     s.row_len[id] = found;
+                    if (fill && s.hist) s.live[id] = ~0u;
                     if (fill && found > cap) atomicExch(ovf, 1);
                 }
                 if (fill)
