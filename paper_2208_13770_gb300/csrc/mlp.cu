@@ -152,7 +152,7 @@ __device__ __forceinline__ double mlp_tile(MlpTile &m, int live, float dy_scale,
 {
     // What bounds a phase is shared memory, 128 bytes a cycle: a warp that
     // takes four units reads each value of the layer below once for four
-    // sums (one unit to a warp and 64 samples: 14,400 cycles a tile, TILEFIG
+    // sums (one unit to a warp and 64 samples: 14,400 cycles a tile, 10,600
     // this way), and the weights four to a load.
     const int lane = threadIdx.x & 31, u = threadIdx.x >> 5;
     const int g4 = (u >> 1) * 4, q = (u & 1) * 32 + lane;   // first unit, sample
@@ -386,7 +386,7 @@ __global__ void k_adam(float *p, const float *part, int nb, float *m, float *v, 
 // batch is enough (the partial sums go to two sets of rows in turn).  The next
 // batch's samples are loaded under this one.  What bounds it is the chain of
 // a batch: six layers' sums of 8 to 64 terms each, a barrier, the partial sums --
-// EPOCHFIG against 38 us with a launch for each batch (34 us, one thread to a
+// 10.8 us for 512 samples, against 37 us with a launch for each batch (one thread to a
 // sample) and one for each step.
 constexpr int kMaxTeam = 64;             // blocks of an epoch's launch
 constexpr unsigned kEpochSpins = 1u << 22;
