@@ -28,6 +28,7 @@ constexpr int kThreads = 256;
 // positions, velocities (policy input) and accelerations.  Launched
 // cooperatively with every block resident.
 // ---------------------------------------------------------------------------
+template <bool kPartial>
 __global__ void __launch_bounds__(kStepMaxThreads, 1)
 k_step(const float4 *__restrict__ pos, const float4 *vel, const float4 *acc,
        const __grid_constant__ DevState sp)
@@ -42,10 +43,10 @@ k_step(const float4 *__restrict__ pos, const float4 *vel, const float4 *acc,
     // check runs
     const unsigned err = c->err;
     if (err & DERR_SYNC) return;   // a barrier failed earlier: the context is unusable
-    const bool inc = s.trigger == LVB_TRIGGER_PARTIAL && !(err & DERR_STORE);
+    const bool inc = kPartial && !(err & DERR_STORE);
     const int step = (int)c->steps + 1, slot = step_slot(step);
     __shared__ __align__(16) lvb_mlp_weights w_sh;
-    const bool net = s.skin_kind == LVB_SKIN_LEARNED;
+    const bool net = kPartial && s.skin_kind == LVB_SKIN_LEARNED;
     if (net) weights_copy_async(&w_sh, s.mlp);
     step_kernel_begin();
     grid_barrier_begin(slot);
@@ -53,7 +54,7 @@ k_step(const float4 *__restrict__ pos, const float4 *vel, const float4 *acc,
     if (s.check_regs) check_pass_regs(s, pos, vel, acc, inc, step, &c->nF_acc[slot]);
     else check_pass_stream(s, pos, vel, acc, inc, step, &c->nF_acc[slot]);
     if (net) weights_copy_wait();
-    if (!finish_step(s, &w_sh, pos, vel, acc, inc, step, slot, t0)) return;
+    if (!finish_step<kPartial>(s, &w_sh, pos, vel, acc, inc, step, slot, t0)) return;
     flush_work(s);
 }
 
@@ -807,6 +808,11 @@ ScanArgs layout_args(lvb_ctx *c)
     return a;
 }
 
+auto step_kernel(const lvb_ctx *c)
+{
+    return c->trigger == LVB_TRIGGER_PARTIAL ? k_step<true> : k_step<false>;
+}
+
 // Blocks of the step kernel for the context's block size: as many as are
 // resident at once (every block must be, the step's barriers wait for all),
 // but no more than the check pass can use.
@@ -816,15 +822,14 @@ int size_step(lvb_ctx *c)
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int smem = c->s.check_regs ? 0 : check_smem_bytes(c->block_threads);
+    const auto fn = step_kernel(c);
     // the attribute belongs to the kernel, for every context of the process:
     // always the largest any block size needs
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_step,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
+        e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  check_smem_bytes(kStepMaxThreads));
     if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step,
-                                                          c->block_threads, smem);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, c->block_threads, smem);
     if (e != cudaSuccess) return from_cuda(e);
     if (per_sm < 1) return LVB_EDEVICE;
     const long long want = (c->n + (long long)c->block_threads * kCheckUnroll - 1) /
@@ -1391,7 +1396,7 @@ int lvb_step(lvb_ctx *c, const float *pos_r, const float *vel, const float *acc)
         if (rc) return rc;
     }
     const cudaError_t e =
-        launch_coop(k_step, dim3(c->step_blocks), dim3(c->block_threads),
+        launch_coop(step_kernel(c), dim3(c->step_blocks), dim3(c->block_threads),
                     c->s.check_regs ? (size_t)0 : (size_t)check_smem_bytes(c->block_threads),
                     c->stream,
                     (const float4 *)pos_r, (const float4 *)vel, a4, c->s);

@@ -560,11 +560,12 @@ __device__ __forceinline__ void advance_pass(const DevState &s, const DemDev &d,
 // (settling 200k 24.6 -> 23.0 us a step).
 static __shared__ DevState s_state;
 
+template <bool kPartial>
 static __device__ __noinline__ bool rest_of_step(const lvb_mlp_weights *w_sh, const float4 *pos,
                                                  const float4 *vel, const float4 *acc, bool inc,
                                                  int step, int slot, unsigned long long t0)
 {
-    return finish_step(s_state, w_sh, pos, vel, acc, inc, step, slot, t0);
+    return finish_step<kPartial>(s_state, w_sh, pos, vel, acc, inc, step, slot, t0);
 }
 
 // `steps` whole DEM steps as one cooperative launch, all blocks resident.
@@ -579,7 +580,7 @@ static __device__ __noinline__ bool rest_of_step(const lvb_mlp_weights *w_sh, co
 // the steps - 1 passes that follow end there, the last forces write d.vel and
 // d.acc.  Those read v* (and w*) as the last pass stored it, so they need no
 // second buffer.
-template <bool kFric>
+template <bool kFric, bool kPartial>
 __global__ void __launch_bounds__(kStepMaxThreads, 1)
 k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
           const __grid_constant__ DemBuffers b, int steps)
@@ -589,7 +590,7 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
     if (err0 & DERR_SYNC) return;   // a barrier failed earlier: the context is unusable
     int step = (int)c->steps, bx = 0, bv = 0;   // the buffers that hold the state
     __shared__ __align__(16) lvb_mlp_weights w_sh;
-    const bool net = s.skin_kind == LVB_SKIN_LEARNED;
+    const bool net = kPartial && s.skin_kind == LVB_SKIN_LEARNED;
     if (net) weights_copy_async(&w_sh, s.mlp);
     step_kernel_begin();
     static_assert(sizeof(DevState) % 4 == 0, "copied in words");
@@ -597,12 +598,12 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
         reinterpret_cast<unsigned *>(&s_state)[t] = reinterpret_cast<const unsigned *>(&s)[t];
     if (step_lead()) atomicAdd(&c->kernels, 1ULL);
     // v* of everyone at every step where the trigger may update anyone
-    const bool star_always = s.trigger != LVB_TRIGGER_PARTIAL || s.early_beta < 1.0f;
+    const bool star_always = !kPartial || s.early_beta < 1.0f;
     for (int k = 1; k <= steps; ++k) {
         const unsigned long long t0 = (s.trace && step_lead()) ? global_ns() : 0ULL;
         const unsigned err = k == 1 ? err0 : *(volatile unsigned *)&c->err;
         const bool store_ok = !(err & DERR_STORE);
-        const bool inc = s.trigger == LVB_TRIGGER_PARTIAL && store_ok;
+        const bool inc = kPartial && store_ok;
         const bool star = star_always || k == steps;
         const int slot = step_slot(++step);
         grid_barrier_begin(slot);
@@ -618,7 +619,7 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
             bx ^= 1;
             bv ^= 1;
         }
-        if (!rest_of_step(&w_sh, b.x[bx], d.vstar, b.a[bv], inc, step, slot, t0)) return;
+        if (!rest_of_step<kPartial>(&w_sh, b.x[bx], d.vstar, b.a[bv], inc, step, slot, t0)) return;
     }
     flush_work(s);
     const unsigned long long t3 = (s.trace && step_lead()) ? global_ns() : 0ULL;
@@ -783,6 +784,13 @@ int launch_phase(dem_ctx *c, int phase)
     return from_cuda(cudaGetLastError());
 }
 
+auto advance_kernel(const dem_ctx *c)
+{
+    if (step_state(c->bp).trigger == LVB_TRIGGER_PARTIAL)
+        return c->d.omega ? k_advance<true, true> : k_advance<false, true>;
+    return c->d.omega ? k_advance<true, false> : k_advance<false, false>;
+}
+
 // Launch shape of k_advance: the broad phase's block size, as many blocks as
 // are resident on the device at once, and no more than have work.
 int advance_shape(dem_ctx *c)
@@ -791,7 +799,7 @@ int advance_shape(dem_ctx *c)
     if (c->shape_of == version) return LVB_OK;
     int threads = 0, dev = 0, sms = 0, per_sm = 0;
     step_shape(c->bp, nullptr, &threads);
-    const void *fn = c->d.omega ? (const void *)k_advance<true> : (const void *)k_advance<false>;
+    const void *fn = (const void *)advance_kernel(c);
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e == cudaSuccess)
@@ -816,10 +824,8 @@ int launch_advance(dem_ctx *c, int steps)
     if (rc) return rc;
     refresh(c);
     const dim3 grid(c->advance_blocks), block(c->advance_threads);
-    return from_cuda(c->d.omega ? launch_coop(k_advance<true>, grid, block, 0, c->stream,
-                                              step_state(c->bp), c->d, c->b, steps)
-                                : launch_coop(k_advance<false>, grid, block, 0, c->stream,
-                                              step_state(c->bp), c->d, c->b, steps));
+    return from_cuda(launch_coop(advance_kernel(c), grid, block, 0, c->stream,
+                                 step_state(c->bp), c->d, c->b, steps));
 }
 
 }  // namespace

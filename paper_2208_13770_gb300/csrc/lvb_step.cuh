@@ -1563,11 +1563,16 @@ static __device__ __noinline__ void full_insert_pass(const DevState &s)
     }
 }
 
+// kDense: with the form for dense cells, for triggers that build whole lists.
+// A re-layout, which a step comes to only when a row outgrew its slack, goes
+// without: the registers that form needs made every step's kernel spill more
+// (see finish_step).
+template <bool kDense>
 static __device__ __noinline__ void all_rows_pass(const DevState &s, int fill, int *ovf,
                                                   bool carry = false)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    if (s.ccap > kTeamSlots) ph_rows_dense(s, fill, t >> 5, nt >> 5, ovf, carry);
+    if (kDense && s.ccap > kTeamSlots) ph_rows_dense(s, fill, t >> 5, nt >> 5, ovf, carry);
     else ph_rows(s, s.n, fill, t >> 5, nt >> 5, ovf, carry);
 }
 
@@ -1651,7 +1656,7 @@ static __device__ __noinline__ bool relayout_pass(const DevState &s)
         save_rows_pass(s);
         if (!grid_barrier(s)) return false;
     }
-    all_rows_pass(s, 0, nullptr);
+    all_rows_pass<false>(s, 0, nullptr);
     if (!grid_barrier(s)) return false;
     const long long need = layout_scan(s, false);
     if (need < 0) return false;
@@ -1666,7 +1671,7 @@ static __device__ __noinline__ bool relayout_pass(const DevState &s)
     if (!grid_barrier(s)) return false;
     if (!store_failed(s)) {
         int unused = 0;
-        all_rows_pass(s, 1, &unused, s.hist != nullptr);
+        all_rows_pass<false>(s, 1, &unused, s.hist != nullptr);
     }
     if (!grid_barrier(s)) return false;
     if (blockIdx.x == 0 && threadIdx.x == 0 && !store_failed(s)) {
@@ -1908,6 +1913,12 @@ __device__ __forceinline__ bool step_lead()
 // updates everyone, for all).  The list is final for every block when it
 // returns true; false: the step was abandoned.  t0: start of the check
 // (trace).
+// kPartial: the trigger is LVB_TRIGGER_PARTIAL; else one of the others.  A kernel
+// holds one of the two only: with both in it, a lone step with nothing flagged
+// after a cold L2 took 12.3 us, not 11.1 (the others: 12.1, not 10.7; 200k
+// spheres), 100 steps of the driver 2,329 us, not 2,288, and a list of 1M
+// spheres built anew 1,009 us, not 926.
+template <bool kPartial>
 __device__ __forceinline__ bool finish_step(const DevState &s, const lvb_mlp_weights *w_sh,
                                             const float4 *pos, const float4 *vel,
                                             const float4 *acc, bool inc, int step, int slot,
@@ -1926,13 +1937,13 @@ __device__ __forceinline__ bool finish_step(const DevState &s, const lvb_mlp_wei
             for (int q = threadIdx.x; q < s.nscenes; q += blockDim.x)
                 s.sc_cnt[spent * s.nscenes + q] = 0;
     }
-    if (inc && nV > 0 && s.early_beta < 1.0f) {
+    if (kPartial && inc && nV > 0 && s.early_beta < 1.0f) {
         early_pass(s, pos, vel, step, nV, &c->nE_acc[slot]);
         if (!grid_barrier(s)) return false;
         nF = nV + *(volatile int *)&c->nE_acc[slot];
     }
     int upd;
-    if (s.trigger == LVB_TRIGGER_PARTIAL) upd = nF;
+    if (kPartial) upd = nF;
     else if (s.trigger == LVB_TRIGGER_GLOBAL) upd = nV ? s.n : 0;
     else upd = s.n;
     unsigned long long t1 = 0;
@@ -1963,8 +1974,8 @@ __device__ __forceinline__ bool finish_step(const DevState &s, const lvb_mlp_wei
         }
     }
     bool changed = false;
-    if (inc) {
-        if (nF > 0) {
+    if (kPartial) {
+        if (inc && nF > 0) {
             if (deferred_update(s)) {
                 update_pass(s, w_sh, nF, pos, vel, acc, step);
                 if (!grid_barrier(s)) return false;
@@ -1978,7 +1989,7 @@ __device__ __forceinline__ bool finish_step(const DevState &s, const lvb_mlp_wei
         if (!grid_barrier(s)) return false;
         full_insert_pass(s);
         if (!grid_barrier(s)) return false;
-        all_rows_pass(s, 1, ovf);
+        all_rows_pass<true>(s, 1, ovf);
         changed = true;
     }
     if (changed) {
@@ -1999,7 +2010,7 @@ __device__ __forceinline__ bool finish_step(const DevState &s, const lvb_mlp_wei
             if (s.trace && lead) trace_add(c, TR_RELAYOUT, t2, global_ns());
         }
     }
-    if (s.log_on) log_pass(s, pos, step);
+    if (kPartial && s.log_on) log_pass(s, pos, step);
     return true;
 }
 
