@@ -204,14 +204,17 @@ __device__ __forceinline__ double mlp_tile(MlpTile &m, int live, float dy_scale,
         }
     }
     __syncthreads();
-    if (u < kTB / 32) {   // the output, one sample to a lane
+    // the output, one sample to a lane, by two warps without units, which sum
+    // the errors in binary64 while the others go back through the layers
+    const int ou = u - NH / 4 * 2;
+    double e = 0.0;
+    if (ou >= 0 && ou < kTB / 32) {
         float y = m.b3;
 #pragma unroll
-        for (int k = 0; k < NH; ++k) y = fmaf(m.w3[k], m.h2T[k][u * 32 + lane], y);
+        for (int k = 0; k < NH; ++k) y = fmaf(m.w3[k], m.h2T[k][ou * 32 + lane], y);
         float dy = 0.0f;
-        double e = 0.0;
-        if (u * 32 + lane < live) {
-            const float lab = m.label[u * 32 + lane];
+        if (ou * 32 + lane < live) {
+            const float lab = m.label[ou * 32 + lane];
             const float r = y - lab;
             float w = 1.0f;   // d(loss)/d(r^2)
             if (rel_floor > 0.0f) {
@@ -221,13 +224,9 @@ __device__ __forceinline__ double mlp_tile(MlpTile &m, int live, float dy_scale,
             dy = dy_scale * w * r;
             e = (double)w * (double)r * (double)r;
         }
-        m.dy[u * 32 + lane] = dy;
-#pragma unroll
-        for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(FULL, e, o);
-        if (lane == 0) m.loss[u] = e;
+        m.dy[ou * 32 + lane] = dy;
     }
     __syncthreads();
-    const double loss = m.loss[0] + m.loss[1];
     if (layers) {
         const float dy = m.dy[q];
 #pragma unroll
@@ -250,8 +249,13 @@ __device__ __forceinline__ double mlp_tile(MlpTile &m, int live, float dy_scale,
         }
 #pragma unroll
         for (int j = 0; j < 4; ++j) m.d1[q][g4 + j] = m.h1T[g4 + j][q] > 0.0f ? g[j] : 0.0f;
+    } else if (ou < kTB / 32) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) e += __shfl_xor_sync(FULL, e, o);
+        if (lane == 0) m.loss[ou] = e;
     }
     __syncthreads();
+    const double loss = m.loss[0] + m.loss[1];
     // The gradients, every sum over the samples in order: warps 0 .. 7 four
     // rows of W2 each, 8 and 9 four columns of W1 each, then b1, b2, w3, b3.
     if (u < 8) {
