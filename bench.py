@@ -6,7 +6,7 @@ Headline workload: 512 independent settling boxes (N per box log-uniform in
 rho 2500, linear spring-dashpot k_n = 1e4, e = 0.7, velocity Verlet
 dt = 1e-6 s, local skin 0.1 d_i) advanced together in one context by the
 library's DEM driver, with the autotuned launch choice.  The run is advanced
-(untimed, 100-step graphs) to step 1,000 - W of its 2,000 steps, W warm-up
+(untimed) to step 1,000 - W of its 2,000 steps, W warm-up
 steps follow, and the K timed steps are steps 1,001 .. 1,000 + K, so any K
 times a representative stretch of the run with list updates in it.  A
 "step" is one DEM step, run phase by phase (integrate, broad phase, narrow
@@ -195,7 +195,7 @@ def _phases(lvb, torch, dem, steps, flush=None, on_step=None):
 
 
 def _advance_to(dem, step, done=0):
-    """Advance the DEM context from step `done` to step `step` (graphs)."""
+    """Advance the DEM context from step `done` to step `step`."""
     if step > done:
         dem.advance(step - done)
 
@@ -434,7 +434,7 @@ def _settling(lvb, torch, steps, warmup, hbm_peak, peak_kind):
     """The 200,000-sphere settling box from step T0_SETTLING: local buffer
     (skin 0.1 d_i) against the paper's global buffer (uniform skin 0.1 x
     mean diameter, any flag rebuilds the whole list), phase by phase, L2
-    flushed before every step; and the driver's fused 100-step graphs."""
+    flushed before every step; and the driver's own steps, 100 to a launch."""
     from paper_2208_13770_gb300 import scenes
     scene = scenes.settling()
     n = scene.n
@@ -479,7 +479,7 @@ def _settling(lvb, torch, steps, warmup, hbm_peak, peak_kind):
     out["speedup_vs_global"] = {
         "local": out["local"]["value"] / out["global_buffer"]["value"],
         "local_early": out["local_early"]["value"] / out["global_buffer"]["value"]}
-    # the driver's own form: one cooperative launch per full DEM step, graphs
+    # the driver's own form: up to 100 full DEM steps in one cooperative launch
     dem = lvb.DEM(scene)
     _advance_to(dem, T0_SETTLING)
     e0 = torch.cuda.Event(enable_timing=True)
@@ -498,7 +498,7 @@ def _settling(lvb, torch, steps, warmup, hbm_peak, peak_kind):
                               "unit": "particle-steps/s (full DEM step)",
                               "ms_per_step": ms / gsteps, "steps": "%d..%d" % (
                                   T0_SETTLING + 1, T0_SETTLING + gsteps),
-                              "l2": "not flushed (100-step graphs)"}
+                              "l2": "not flushed (100 steps to a launch)"}
     return out
 
 
@@ -513,7 +513,7 @@ def _drum_scene(n=DRUM_N, length=0.20):
 
 
 def _spun_up(lvb, sc, steps):
-    """The drum after `steps` steps of the driver (graphs), as a new scene
+    """The drum after `steps` steps of the driver, as a new scene
     object (positions and velocities), for runs that start from it."""
     dem = lvb.DEM(sc)
     dem.advance(steps)
@@ -529,7 +529,7 @@ def _spun_up(lvb, sc, steps):
 def _drum(lvb, torch, hbm_peak, peak_kind, k_sweep=(0, 50, 100, 200, 400, 1000, 5000)):
     """The 2,000,000-sphere drum (lognormal radii, 0.20 m long, bed turned
     30 degrees, 5% of the particles in a dilute cascading layer): spin-up of
-    DRUM_SPINUP steps, then DRUM_STEPS full steps in graphs; the broad phase
+    DRUM_SPINUP steps, then DRUM_STEPS full steps; the broad phase
     phase by phase over 500 steps; a K sweep of the paper's rule; and the
     stencil's reach bounds against a plain 27-cell stencil."""
     sc = _drum_scene()
@@ -540,7 +540,7 @@ def _drum(lvb, torch, hbm_peak, peak_kind, k_sweep=(0, 50, 100, 200, 400, 1000, 
                        "0.35, clipped [0.4, 3] mm), bed turned 30 deg with 5%% in a dilute "
                        "cascading layer, 10 rpm, dt 1e-6 s; %d steps of spin-up, then the "
                        "timed steps" % (n, DRUM_SPINUP), "n": n}
-    # full steps, graphs
+    # full steps of the driver
     dem = lvb.DEM(mid)
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
@@ -620,7 +620,7 @@ LEARN_STEPS = 1500      # steps of the logged training run and of each timed run
 
 
 def _timed_advance(lvb, torch, scene, kind, value, mlp=None, log=None, steps=LEARN_STEPS):
-    """Advance a fresh DEM context `steps` steps in 100-step graphs; returns
+    """Advance a fresh DEM context `steps` steps, 100 to a launch; returns
     full-step particle-steps/s, updates/step, mean entries, rebuild steps
     (and the rebuild-log samples when log is a horizon)."""
     dem = lvb.DEM(scene, skin_kind=kind, skin_value=value, mlp=mlp)
@@ -728,7 +728,7 @@ def _learned(lvb, torch):
 
 def _friction(lvb, torch):
     """Friction with contact history on the 1,000,000-sphere drum (mu 0.5,
-    k_t = 2/7 k_n, gamma_t = 0.5 gamma_n): full DEM steps in graphs with and
+    k_t = 2/7 k_n, gamma_t = 0.5 gamma_n): full DEM steps with and
     without friction from the same state, and the broad phase alone phase by
     phase with the history on (flagged rows edited in place) and off."""
     from paper_2208_13770_gb300 import scenes
@@ -757,7 +757,7 @@ def _friction(lvb, torch):
         dem.close()
         out[name] = {"full_step_value": sc.n * 1000 / (ms * 1e-3),
                      "full_step_us": 1e3 * ms / 1000,
-                     "unit": "particle-steps/s (full DEM step, graphs)",
+                     "unit": "particle-steps/s (full DEM step)",
                      "broad_us_per_step": 1e3 * ph[1] / 300,
                      "forces_us_per_step": 1e3 * ph[2] / 300,
                      "flagged_per_step": _diff(s0, s1, "flagged_total") / 300}

@@ -128,7 +128,8 @@ int lvb_mlp_grad(const float *samples, int64_t n, const float *params, const flo
  *   y_range     : host out, {y_lo, y_hi} from the labels' mean m and
  *                 standard deviation sd: y_lo = m / 16, y_hi = m + 4 sd.
  *   losses      : host out, mean loss of every epoch (epochs entries).
- * Synchronises.  Errors: EINVAL, ENOMEM, EDEVICE.
+ * Synchronises.  Errors: EINVAL, ENOMEM, EDEVICE, ETIMEOUT (the blocks of an
+ * epoch's launch waited too long for one another).
  */
 int lvb_mlp_train(const float *samples, int64_t n, int32_t epochs, int32_t batch, float lr,
                   uint64_t seed, int32_t loss_kind, float *params, float *mu, float *isd,

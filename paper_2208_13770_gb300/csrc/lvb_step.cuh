@@ -1006,7 +1006,8 @@ __device__ __forceinline__ void ph_rows(const DevState &s, int nitems, int fill,
 // 230 candidates a row for 6 partners, the whole list at every step: 1,421 us
 // with a warp to a row and a flattened run of its candidates, 1,360 with a
 // warp to a row and its cells one after another at 925 instructions a row,
-// 899 this way at 590; two or four rows tested together: 928 and 960).
+// 899 this way at 590; two or four rows tested together: 928 and 960; 809 in a
+// kernel that holds no partial rebuild).
 // Warps w0, w0 + wstride, ... take the cells round and round, the next 32 slots
 // of the same cell by another warp.
 __device__ __forceinline__ void ph_rows_dense(const DevState &s, int fill, int w0, int wstride,
