@@ -991,7 +991,7 @@ int copy_out(lvb_ctx *c, void *dst, const void *src, size_t bytes)
 // kernel that looks at the errors itself (200k flags: two waits, 20 us, less).
 int copy_checked(lvb_ctx *c, void *dst, const void *src, size_t bytes)
 {
-    if (((uintptr_t)dst & 3u) || !on_device(dst)) {
+    if (!on_device(dst)) {
         int rc = sync_counters(c);
         if (!rc) rc = copy_out(c, dst, src, bytes);
         return rc ? rc : from_cuda(cudaStreamSynchronize(c->stream));
@@ -1818,12 +1818,16 @@ int sync_counters_of(lvb_ctx *c, const DevCounters **host)
 
 bool on_device(const void *p)
 {
+    if ((uintptr_t)p & 3u) return false;   // copies take any address, kernels do not
     cudaPointerAttributes a{};
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();   // an unknown pointer: host memory
         return false;
     }
-    return a.type == cudaMemoryTypeDevice || a.type == cudaMemoryTypeManaged;
+    int dev = -1;
+    return a.type == cudaMemoryTypeManaged ||
+           (a.type == cudaMemoryTypeDevice && cudaGetDevice(&dev) == cudaSuccess &&
+            a.device == dev);
 }
 
 int grow_stores_if_asked(lvb_ctx *c)

@@ -328,7 +328,8 @@ cudaStream_t step_stream(lvb_ctx *c);
 // Waits for the context's stream and reads its counters back: the sticky device
 // error, and the counters through *host (valid until the next such call).
 int sync_counters_of(lvb_ctx *c, const DevCounters **host);
-// Whether p is memory that kernels may write in place (device or managed).
+// Whether p is memory that kernels may write in place, in words of four bytes:
+// of the current device or managed, and on such an address.
 bool on_device(const void *p);
 
 // Changes whenever the step kernel's arguments or launch shape change

@@ -104,3 +104,35 @@ def test_lists_match_brute_force(n, crowd, where):
                                  ctypes.byref(got)) == lvb.LVB_ECAPACITY
         assert np.array_equal(rows.cpu().numpy(), ptr) and int((col != -7).sum()) == 0
     ctx.close()
+
+
+def test_device_arrays_off_their_words():
+    """Device arrays at an odd address hold the same bytes as aligned ones."""
+    lvb = _lvb()
+    n = 257
+    pos, side = _cloud(n, 60, 11)
+    x = torch.from_numpy(pos).cuda()
+    ctx = lvb.LVB(x, (0, 0, 0), (side, side, side), lvb.LVB_SKIN_DIAMETER_FACTOR, 0.1, 1e-6)
+    want = _brute(pos, 0.1, ctx.stats()["rnl_max"])
+    m = len(want)
+
+    def buf(words):
+        return torch.zeros(4 * words + 4, dtype=torch.uint8, device="cuda")[1:4 * words + 1]
+
+    def words(t):
+        return np.frombuffer(t.cpu().numpy().tobytes(), np.int32)
+
+    got = ctypes.c_int64(-1)
+    a, b, rows, col = buf(m), buf(m), buf(n + 1), buf(2 * m)
+    assert lvb.lvb_get_pairs_ij(ctx.ctx, a.data_ptr(), b.data_ptr(), m, ctypes.byref(got)) == 0
+    assert words(a).tolist() == [p[0] for p in want] and words(b).tolist() == [p[1] for p in want]
+    assert lvb.lvb_get_pairs(ctx.ctx, rows.data_ptr(), col.data_ptr(), 2 * m,
+                             ctypes.byref(got)) == 0
+    i2, j2 = (np.array([p[k] for p in want] + [p[1 - k] for p in want]) for k in (0, 1))
+    assert np.array_equal(words(col), j2[np.lexsort((j2, i2))])
+    assert np.array_equal(np.diff(words(rows)), np.bincount(i2, minlength=n))
+    ref, ref_al = buf(4 * n), torch.zeros(4 * n, dtype=torch.float32, device="cuda")
+    assert lvb.lvb_get_ref(ctx.ctx, ref.data_ptr()) == 0
+    assert lvb.lvb_get_ref(ctx.ctx, ref_al.data_ptr()) == 0
+    assert ref.cpu().numpy().tobytes() == ref_al.cpu().numpy().tobytes()
+    ctx.close()
