@@ -557,7 +557,9 @@ __device__ __forceinline__ void advance_pass(const DevState &s, const DemDev &d,
 // not displace the pass's.  To a call the kernel's parameter is memory like
 // any other, cached in an L1 that every grid barrier empties, so the phases
 // after the pass read the context's state from a copy in shared memory
-// (settling 200k 24.6 -> 23.0 us a step).
+// (settling 200k 24.6 -> 23.0 us a step).  Some threads fill it and all read
+// it, from before the first grid barrier on (a warp without particles comes
+// straight to it), so the block barrier that follows the filling publishes it.
 static __shared__ DevState s_state;
 
 template <bool kPartial>
@@ -596,6 +598,7 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
     static_assert(sizeof(DevState) % 4 == 0, "copied in words");
     for (int t = threadIdx.x; t < (int)(sizeof(DevState) / 4); t += blockDim.x)
         reinterpret_cast<unsigned *>(&s_state)[t] = reinterpret_cast<const unsigned *>(&s)[t];
+    __syncthreads();   // s_state
     if (step_lead()) atomicAdd(&c->kernels, 1ULL);
     // v* of everyone at every step where the trigger may update anyone
     const bool star_always = !kPartial || s.early_beta < 1.0f;
