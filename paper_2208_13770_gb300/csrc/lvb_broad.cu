@@ -44,7 +44,7 @@ k_step(const float4 *__restrict__ pos, const float4 *vel, const float4 *acc,
     const unsigned err = c->err;
     if (err & DERR_SYNC) return;   // a barrier failed earlier: the context is unusable
     const bool inc = kPartial && !(err & DERR_STORE);
-    const int step = (int)c->steps + 1, slot = step_slot(step);
+    const int step = next_step((unsigned)c->steps), slot = step_slot(step);
     __shared__ __align__(16) lvb_mlp_weights w_sh;
     const bool net = kPartial && s.skin_kind == LVB_SKIN_LEARNED;
     if (net) weights_copy_async(&w_sh, s.mlp);
@@ -1216,11 +1216,12 @@ static int init_impl(lvb_ctx **out, int nscenes, const int64_t *offsets, int64_t
     if (e == cudaSuccess) e = dalloc(&s.bits, c->nwords);
     if (e == cudaSuccess) e = dalloc(&s.fid, n);
     if (nscenes > 1) {
-        if (e == cudaSuccess) e = dalloc(&s.sc_cnt, 3LL * nscenes);
+        if (e == cudaSuccess) e = dalloc(&s.sc_cnt, (long long)kStepSlots * nscenes);
         if (e == cudaSuccess) e = dalloc(&s.sfid, n);
         if (e == cudaSuccess) e = dalloc(&s.sfref, n);
         if (e == cudaSuccess) e = dalloc(&s.fsc, n);
-        if (e == cudaSuccess) e = cudaMemsetAsync(s.sc_cnt, 0, sizeof(int) * 3 * nscenes, st);
+        if (e == cudaSuccess)
+            e = cudaMemsetAsync(s.sc_cnt, 0, sizeof(int) * kStepSlots * nscenes, st);
     }
     if (e == cudaSuccess) e = dalloc(&s.row_off, n);
     if (e == cudaSuccess) e = dalloc(&s.row_len, n);

@@ -590,7 +590,8 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
     DevCounters *c = s.cnt;
     const unsigned err0 = c->err;
     if (err0 & DERR_SYNC) return;   // a barrier failed earlier: the context is unusable
-    int step = (int)c->steps, bx = 0, bv = 0;   // the buffers that hold the state
+    const unsigned done = (unsigned)c->steps;
+    int bx = 0, bv = 0;   // the buffers that hold the state
     __shared__ __align__(16) lvb_mlp_weights w_sh;
     const bool net = kPartial && s.skin_kind == LVB_SKIN_LEARNED;
     if (net) weights_copy_async(&w_sh, s.mlp);
@@ -608,7 +609,7 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
         const bool store_ok = !(err & DERR_STORE);
         const bool inc = kPartial && store_ok;
         const bool star = star_always || k == steps;
-        const int slot = step_slot(++step);
+        const int step = next_step(done + k - 1), slot = step_slot(step);
         grid_barrier_begin(slot);
         int *nF_acc = &c->nF_acc[slot];
         if (k == 1) {

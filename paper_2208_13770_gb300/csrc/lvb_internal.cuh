@@ -21,6 +21,7 @@
 
 #include "lvb.h"
 #include "lvb_mlp.h"
+#include "step_slots.cuh"
 
 #include <cuda_bf16.h>
 
@@ -38,16 +39,17 @@ enum TraceSlot {
 
 struct DevCounters {
     int nF;            // flagged at the last step (final)
-    int nF_acc[3];     // flagged count while the check runs (slot: step_slot)
-    int nE_acc[3];     // updated early beyond them (LVB_OPT_EARLY)
-    int next_patch[3]; // patches handed out beyond the first of each team
-    int ovf[3];        // a row outgrew its capacity (slot: step_slot)
+    // by step_slot:
+    int nF_acc[kStepSlots];      // flagged count while the check runs
+    int nE_acc[kStepSlots];      // updated early beyond them (LVB_OPT_EARLY)
+    int next_patch[kStepSlots];  // patches handed out beyond the first of each team
+    int ovf[kStepSlots];         // a row outgrew its capacity
     int row_overflow;  // same, for the separate full-build kernels
     int force_relayout;  // the next step that rebuilds rows re-lays them out (test hook)
     unsigned err;      // sticky DERR_* bits
     int last_flagged;
     int last_updated;
-    unsigned long long bar_cnt[3];  // grid-barrier arrivals in the step kernel (slot: step_slot)
+    unsigned long long bar_cnt[kStepSlots];  // grid-barrier arrivals in the step kernel (by step_slot)
     long long steps;
     long long rebuild_steps;
     long long flagged_total;

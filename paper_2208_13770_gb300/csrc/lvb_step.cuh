@@ -62,7 +62,7 @@ struct DevState {
     // many scenes: the flagged particles of scene q also sit in its own
     // segment [first_q, first_q + sc_cnt[slot][q]) of sfid / sfref, so the
     // direct flagged test scans only its scene (null with one scene)
-    int *sc_cnt;      // 3 x nscenes counters (by step_slot)
+    int *sc_cnt;      // kStepSlots x nscenes counters (by step_slot)
     int *sfid;
     float4 *sfref;
     int *fsc;         // scene of each flagged particle, same order as fid
@@ -130,15 +130,6 @@ struct DevState {
 
 // gate modes of the separate full-build kernels (init, store growth)
 enum Gate { GATE_OVERFLOW = 1, GATE_ANY_FLAG = 2, GATE_ALWAYS = 3 };
-
-// Per-step counts live in three slots, step_slot(step) at a step: the steps
-// of one kernel follow one another with as little as one grid barrier
-// between them, so a block may already count the next step while another
-// still reads this one's counts, and only the slot of the step before is
-// free for everyone.  Each step clears that one after its first barrier,
-// which is the slot of the step after the next.
-__device__ __forceinline__ int step_slot(int step) { return step % 3; }
-__device__ __forceinline__ int spent_slot(int slot) { return slot == 0 ? 2 : slot - 1; }
 
 __device__ __forceinline__ const SceneGeom &geom_of(const DevState &s, int i)
 {
@@ -1932,7 +1923,7 @@ __device__ __forceinline__ bool finish_step(const DevState &s, const lvb_mlp_wei
     if (!grid_barrier(s)) return false;
     const int nV = *(volatile int *)&c->nF_acc[slot];   // violations of Eq. update
     int nF = nV;                                         // particles updated
-    if (blockIdx.x == 0) {   // the spent slot, which the step after the next counts on
+    if (blockIdx.x == 0) {   // the spent slot, for a later step to count on
         if (threadIdx.x == 0) c->bar_cnt[spent] = 0;
         if (s.sc_cnt)
             for (int q = threadIdx.x; q < s.nscenes; q += blockDim.x)
