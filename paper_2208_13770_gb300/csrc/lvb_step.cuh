@@ -732,18 +732,13 @@ __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int 
     // the first records of the flagged list.  Many scenes: the scene's own
     // segment of the flagged particles (scenes share one coordinate frame,
     // so the global list would also hold far-away twins)
-    auto listed = [&](int kk, float4 &r, int &j) {
-        r = make_float4(0.f, 0.f, 0.f, 0.f);
-        j = -1;
-        if (kk < m_dir) {
-            const bool own = s.sc_cnt != nullptr;
-            r = own ? s.sfref[g.first + kk] : s.fref[kk];
-            j = own ? s.sfid[g.first + kk] : s.fid[kk];
-        }
-    };
-    float4 rf0;
-    int jf0;
-    listed(e0, rf0, jf0);
+    const int seg = s.sc_cnt ? g.first : 0;
+    float4 rf0 = make_float4(0.f, 0.f, 0.f, 0.f);
+    int jf0 = -1;
+    if (e0 < m_dir) {
+        rf0 = (s.sc_cnt ? s.sfref : s.fref)[seg + e0];
+        jf0 = (s.sc_cnt ? s.sfid : s.fid)[seg + e0];
+    }
     if (tw == 0 && lane == 0 && m_dir) atomicAdd(&s_work[1], (unsigned long long)m_dir);
     // whether old entry j leaves row i, and (jr, at sp) whether i leaves row j:
     // the partner's flag word, reference state, radius and row bounds are
@@ -810,9 +805,9 @@ __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int 
             }
         }
     };
-    // the flagged partners of the direct test
+    // the flagged partners of the direct test (all of this scene)
     auto flagged = [&](int j, float4 r) {
-        bool take = j >= g.first && j < g.first + g.count && j != i && pair_hit(qn, r);
+        bool take = pair_hit(qn, r) && j >= 0 && j != i;
         if (kHist) take = take && !pair_hit(s.oref[k], s.pold[j]);
         append(take, j);
     };
@@ -872,12 +867,17 @@ __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int 
     do take_up();   // (once in any case: the removals of the old row)
     while (n_noted > 0);
     // the rest of the flagged list, kDirectUnroll records per lane in flight
+    // and nothing else to load
+    const float4 *lst = (s.sc_cnt ? s.sfref : s.fref) + seg;
+    const int *ids = (s.sc_cnt ? s.sfid : s.fid) + seg;
     for (int b0 = per + tw * 32 * kDirectUnroll; b0 < m_dir; b0 += per * kDirectUnroll) {
         float4 rf[kDirectUnroll];
         int jf[kDirectUnroll];
 #pragma unroll
         for (int u = 0; u < kDirectUnroll; ++u) {
-            listed(b0 + u * 32 + lane, rf[u], jf[u]);
+            const int kk = b0 + u * 32 + lane;
+            rf[u] = kk < m_dir ? lst[kk] : make_float4(0.f, 0.f, 0.f, 0.f);
+            jf[u] = kk < m_dir ? ids[kk] : -1;
         }
 #pragma unroll
         for (int u = 0; u < kDirectUnroll; ++u) flagged(jf[u], rf[u]);
