@@ -171,7 +171,7 @@ k_rows(DevState s, int gate, int fill, int carry = 0)
     count_kernel(s);
     tr_enter(s, TR_ROWS);
     const int w0 = (blockIdx.x * kThreads + threadIdx.x) >> 5, nw = (gridDim.x * kThreads) >> 5;
-    if (s.ccap > kTeamSlots)
+    if (s.dense_rows)
         ph_rows_dense(s, fill, w0, nw, &s.cnt->row_overflow, carry != 0);
     else ph_rows(s, nitems, fill, w0, nw, &s.cnt->row_overflow, carry != 0);
     tr_exit(s, TR_ROWS);
@@ -330,13 +330,36 @@ __global__ void k_radius_store(const float4 *__restrict__ pos, int n, float *rad
         rad[i] = pos[i].w;
 }
 
-__global__ void k_max_int(const int *v, long long n, int *out)
+// How full the cells are: the fullest, those that hold anyone, and the sum of
+// the squares (so, over n, the particles in a particle's cell).
+struct Occupancy {
+    int most;
+    unsigned occupied;
+    unsigned long long squares;
+};
+
+__global__ void k_occupancy(const int *cnt, long long ncells, Occupancy *out)
 {
     int m = 0;
-    for (long long c = blockIdx.x * kThreads + threadIdx.x; c < n; c += (long long)gridDim.x * kThreads)
-        m = max(m, v[c]);
-    for (int o = 16; o; o >>= 1) m = max(m, __shfl_xor_sync(FULL, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(out, m);
+    unsigned k = 0;
+    unsigned long long q = 0;
+    for (long long c = blockIdx.x * kThreads + threadIdx.x; c < ncells;
+         c += (long long)gridDim.x * kThreads) {
+        const int v = cnt[c];
+        m = max(m, v);
+        k += v > 0;
+        q += (unsigned long long)v * (unsigned)v;
+    }
+    for (int o = 16; o; o >>= 1) {
+        m = max(m, __shfl_xor_sync(FULL, m, o));
+        k += __shfl_xor_sync(FULL, k, o);
+        q += __shfl_xor_sync(FULL, q, o);
+    }
+    if ((threadIdx.x & 31) == 0 && k) {
+        atomicMax(&out->most, m);
+        atomicAdd(&out->occupied, k);
+        atomicAdd(&out->squares, q);
+    }
 }
 
 // Live entries of the list (rows hold -1 where a pair was removed).
@@ -851,6 +874,24 @@ int sync_counters(lvb_ctx *c)
     return from_derr(c->cnt_h->err);
 }
 
+// Reads how full the cells are (cell_cnt) and chooses the rows' form by it.
+// Waits for the stream.
+int read_occupancy(lvb_ctx *c, Occupancy *o)
+{
+    Occupancy *d = reinterpret_cast<Occupancy *>(c->scratch);
+    cudaError_t e = cudaMemsetAsync(d, 0, sizeof(Occupancy), c->stream);
+    if (e != cudaSuccess) return from_cuda(e);
+    k_occupancy<<<grid_for(c->ncells, kThreads, 4 * kNumSMs), kThreads, 0, c->stream>>>(
+        c->s.cell_cnt, c->ncells, d);
+    e = cudaMemcpyAsync(o, d, sizeof(Occupancy), cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (e != cudaSuccess) return from_cuda(e);
+    c->s.dense_rows = c->n >= (int64_t)kDenseRows * o->occupied;
+    c->s.dense_many = c->s.dense_rows &&
+                      o->squares >= (unsigned long long)kDenseMany * (unsigned long long)c->n;
+    return LVB_OK;
+}
+
 // Grows the row store and/or the cell slots when a kernel asked for it
 // (over 75% full), then rebuilds the cells and rows from the current
 // reference state -- the list is a function of that state alone, so the
@@ -883,6 +924,9 @@ int grow_if_asked(lvb_ctx *c)
         k_cells_clear<<<grid_for(c->ncells, kThreads, 4 * kNumSMs), kThreads, 0, st>>>(
             s, GATE_ALWAYS);
         k_cells_insert<<<items_grid(c), kThreads, 0, st>>>(s, GATE_ALWAYS, 0);
+        Occupancy occ;
+        const int rc = read_occupancy(c, &occ);
+        if (rc) return rc;
     }
     // rows: count, then a store with room to grow, then fill
     k_rows<<<rows_grid(c), kThreads, 0, st>>>(s, GATE_ALWAYS, 0);
@@ -1283,17 +1327,13 @@ static int init_impl(lvb_ctx **out, int nscenes, const int64_t *offsets, int64_t
     // and room for a dense packing of mean-volume particles)
     cudaMemsetAsync(s.cell_cnt, 0, sizeof(int) * ncells, st);
     k_cells_insert<<<gi, kThreads, 0, st>>>(s, GATE_ALWAYS, 1);
-    cudaMemsetAsync(c->scratch, 0, sizeof(int), st);
-    k_max_int<<<grid_for(ncells, kThreads, 4 * kNumSMs), kThreads, 0, st>>>(s.cell_cnt, ncells,
-                                                                           (int *)c->scratch);
-    int maxocc = 0;
-    e = cudaMemcpyAsync(&maxocc, c->scratch, sizeof(int), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-    if (e != cudaSuccess) return fail(from_cuda(e));
+    Occupancy occ;
+    rc = read_occupancy(c, &occ);
+    if (rc) return fail(rc);
     {
         const double vmean = 4.0 / 3.0 * M_PI * r3mean;
         const double dense = 0.74 * Lmax * Lmax * Lmax / std::max(vmean, 1e-30);
-        long long cap = std::max<long long>(2LL * maxocc + 8, 32);
+        long long cap = std::max<long long>(2LL * occ.most + 8, 32);
         cap = std::max<long long>(cap, (long long)std::min(dense * 0.5, 4096.0));
         cap = (cap + 31) / 32 * 32;
         cap = std::min<long long>(cap, 1 << 16);

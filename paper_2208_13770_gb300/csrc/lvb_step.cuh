@@ -104,6 +104,8 @@ struct DevState {
                           // 0 the bulk-copy ring (LVB_OPT_CHECK_LOADS)
     int reach;            // stencil cells skipped by distance (LVB_OPT_STENCIL_REACH):
                           // 0 none, 1 by the cap H, 2 by H and the cell's own bound
+    int dense_rows;       // the cells that hold anyone hold kDenseRows each, in the mean
+    int dense_many;       // and a particle's cell kDenseMany
     // second destination of this step's flag words and flagged count
     // (lvb_step_host: a staging slot copied out while the next step runs),
     // or null
@@ -589,7 +591,20 @@ __device__ __forceinline__ void team_sync(const Team &t)
 // context's counters by thread 0 once per kernel
 static __shared__ unsigned long long s_work[3];
 
-constexpr int kTeamSlots = 64;   // slots per cell above which cells count as dense
+// Which form the rows take (DevState::dense_rows, dense_many).  The forms for
+// dense cells pay for every cell that holds anyone, the others for every
+// candidate, so the line lies at so many particles to an occupied cell, not at
+// the slots a cell has (one crowded cell, or a growth, gives all cells many).
+// 200k spheres, means of 1.9, 4.0, 7.5, 11.8, 14.5, 25 (whole list, us; a warp
+// to a row): 802, 459, 254, 267, 239, 239 against 211, 217, 201, 272, 274, 335.
+// Patches by teams of warps are even at 3 to 10 (28 to 30 us a step with 20 or
+// 200 flagged, either way) and gain from there (30.8 -> 28.3 us at 41, 34.2 ->
+// 28.4 at 91); with so many flagged that a patch has a single warp, its cells
+// one after another, only where the particles see many others: at 27, 47, 57
+// and 94 to the cell of a particle, 67, 67, 72 and 72 us against 60, 64, 73 and
+// 75 with 6,000 flagged.
+constexpr int kDenseRows = 12;   // particles to an occupied cell, from which rows are dense
+constexpr int kDenseMany = 48;   // particles in a particle's cell, from which many patches are
 
 constexpr int kNoted = 64;   // candidates a warp notes before it takes them up
 static __shared__ __align__(16) int2 s_noted[kStepMaxThreads / 32][kNoted];
@@ -634,11 +649,11 @@ static __shared__ unsigned s_team_free[kStepMaxThreads / 32]; // its free slots 
 // phase, per step, before and after: 2M drum 10k flagged 79 -> 50 us, 1M drum
 // with friction 45 -> 20 us, 6.2M batch 13.2 -> 11.8 us, 2k gas 7.4 -> 5.6 us.
 //
-// kDense (cells of more than kTeamSlots slots): the candidates are taken cell
-// by cell, the cells shared out among the warps of a team; otherwise the team
-// is one warp, and the few candidates of the 27 cells are taken as one run,
-// each lane finding its cell by a shuffle search (which, at 32 candidates a
-// time, would be most of the work in a dense bed).
+// kDense (partial_pass says when): the candidates are taken cell by cell, the
+// cells shared out among the warps of a team; otherwise the team is one warp,
+// and the few candidates of the 27 cells are taken as one run, each lane finding
+// its cell by a shuffle search (which, at 32 candidates a time, would be most of
+// the work in a dense bed).
 template <bool kHist, bool kDense>
 __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int k, int nF,
                                               bool direct, int slot, int *ovf)
@@ -987,7 +1002,7 @@ __device__ __forceinline__ void ph_rows(const DevState &s, int nitems, int fill,
     }
 }
 
-// The same in dense cells (more than kTeamSlots slots): a warp takes 32 slots
+// The same in dense cells (DevState::dense_rows): a warp takes 32 slots
 // of a cell at a time, one row to a lane, and each of the 27 cells around it in
 // turn.  One ballot tells which of the rows reach that cell at all; its
 // candidates are held 32 at a time, one to a lane, and every such row is
@@ -1564,7 +1579,7 @@ static __device__ __noinline__ void all_rows_pass(const DevState &s, int fill, i
                                                   bool carry = false)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    if (kDense && s.ccap > kTeamSlots) ph_rows_dense(s, fill, t >> 5, nt >> 5, ovf, carry);
+    if (kDense && s.dense_rows) ph_rows_dense(s, fill, t >> 5, nt >> 5, ovf, carry);
     else ph_rows(s, s.n, fill, t >> 5, nt >> 5, ovf, carry);
 }
 
@@ -1849,21 +1864,23 @@ static __device__ __noinline__ void move_pass(const DevState &s, int nF)
 // flagged particles: moves and patches in one phase, on different warps (the
 // patches skip the flagged particles in the cells and test them directly);
 // more: the moves first and a barrier, then the patches on final cells.
-// In dense cells (more than kTeamSlots slots) a team has as many warps (1, 4,
-// 8, 16 or 32) as leave every patch a team and every move a warp of its own
-// (1M drum with friction, 930 flagged: rebuild 41 us with single warps, 25 us
-// with teams of four, before the candidates were noted).  In sparse cells a
-// row has some 20 candidates, which one warp loads at once, and the team's
-// barriers only add to its chain (settling 200k: 23.8 -> 25.3 us a step).
+// In dense cells (dense_rows) a team has as many warps (1, 4, 8, 16 or 32) as
+// leave every patch a team and every move a warp of its own (1M drum with
+// friction, 930 flagged: rebuild 41 us with single warps, 25 us with teams of
+// four, before the candidates were noted); where that is one warp, the form for
+// dense cells is taken with dense_many only.  In sparse cells a row has some 20
+// candidates, which one warp loads at once, and the team's barriers only add to
+// its chain (settling 200k: 23.8 -> 25.3 us a step).
 // Returns false when the step must be abandoned.
 __device__ __forceinline__ bool partial_pass(const DevState &s, int nF, int slot, int *ovf)
 {
     const int wpb = blockDim.x >> 5, nw = gridDim.x * wpb;
-    const bool direct = nF <= s.direct_max, dense = s.ccap > kTeamSlots;
+    const bool direct = nF <= s.direct_max;
     int lg = 0;   // log2 of the team's size
-    if (dense && nF <= nw)   // (no product beyond 32 bits)
+    if (s.dense_rows && nF <= nw)   // (no product beyond 32 bits)
         for (int t = 2; t <= 5; ++t)
             if ((1 << t) <= wpb && nF * ((1 << t) + (direct ? 1 : 0)) <= nw) lg = t;
+    const bool dense = lg > 0 || s.dense_many;
     if (!direct) {
         move_pass(s, nF);
         if (!grid_barrier(s)) return false;
