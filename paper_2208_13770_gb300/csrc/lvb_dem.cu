@@ -289,13 +289,17 @@ __device__ __forceinline__ bool add_contact(const DemDev &d, const Star &star, c
 // is read four entries at a time (rows start on 16 bytes) and the four
 // partners' positions together, so that a row of up to four costs two memory
 // latencies; only the few that may touch are taken up again, one after
-// another (their positions then come from the L1).
+// another (their positions then come from the L1).  kMany: entry by entry, with
+// the next partner's position in flight.  Where many touch, taking those up again
+// saves no turns, and what bounds the loop is the gathers: one of 32 partners in
+// no order is some 30 passes through the L1 (1M packed spheres, 3 contacts each,
+// a launch of one step: 103 -> 87 us; 1M settling ones, next to none: 54 -> 59 us).
 // With friction, an entry out of contact keeps no spring.  Most had none
 // already, so the records are not written over and over (16 bytes for each of
 // the four entries in six of a drum's row): live[i] has a bit for each of the
 // row's first 32 entries whose record may be other than zero, and only those
 // are cleared (1M drum, a pass over the particles: 111 -> 80 us).
-template <bool kFric, class Star>
+template <bool kFric, bool kMany, class Star>
 __device__ __forceinline__ void row_forces(const DemDev &d, const float4 *X, const Star &star,
                                            const Star &spin, float4 xi, float4 vi, int i, int off,
                                            int len, float F[3], float T[3])
@@ -305,23 +309,37 @@ __device__ __forceinline__ void row_forces(const DemDev &d, const float4 *X, con
     unsigned live = live0;
     for (int e0 = 0; e0 < len; e0 += 4) {
         const int4 j4 = *reinterpret_cast<const int4 *>(d.rows.col + off + e0);
-        float4 xj[4];
-        xj[0] = j4.x >= 0 ? X[j4.x] : zero;
-        xj[1] = j4.y >= 0 ? X[j4.y] : zero;
-        xj[2] = j4.z >= 0 ? X[j4.z] : zero;
-        xj[3] = j4.w >= 0 ? X[j4.w] : zero;
-        unsigned m = 0;
-        if (j4.x >= 0 && may_touch(xi, xj[0])) m |= 1u;
-        if (j4.y >= 0 && may_touch(xi, xj[1])) m |= 2u;
-        if (j4.z >= 0 && may_touch(xi, xj[2])) m |= 4u;
-        if (j4.w >= 0 && may_touch(xi, xj[3])) m |= 8u;
         unsigned in = 0;   // entries in contact
-        while (m) {
-            const int u = __ffs(m) - 1;
-            m &= m - 1;
-            const int j = u < 2 ? (u == 0 ? j4.x : j4.y) : (u == 2 ? j4.z : j4.w);
-            if (add_contact<kFric>(d, star, spin, xi, vi, i, off + e0 + u, j, X[j], F, T))
-                in |= 1u << u;
+        if (kMany) {
+            float4 xj = j4.x >= 0 ? X[j4.x] : zero;
+#pragma unroll 1
+            for (int u = 0; u < 4; ++u) {
+                const int j = u < 2 ? (u == 0 ? j4.x : j4.y) : (u == 2 ? j4.z : j4.w);
+                const int after = u < 2 ? (u == 0 ? j4.y : j4.z) : (u == 2 ? j4.w : -1);
+                const float4 xn = after >= 0 ? X[after] : zero;
+                if (j >= 0 &&
+                    add_contact<kFric>(d, star, spin, xi, vi, i, off + e0 + u, j, xj, F, T))
+                    in |= 1u << u;
+                xj = xn;
+            }
+        } else {
+            float4 xj[4];
+            xj[0] = j4.x >= 0 ? X[j4.x] : zero;
+            xj[1] = j4.y >= 0 ? X[j4.y] : zero;
+            xj[2] = j4.z >= 0 ? X[j4.z] : zero;
+            xj[3] = j4.w >= 0 ? X[j4.w] : zero;
+            unsigned m = 0;
+            if (j4.x >= 0 && may_touch(xi, xj[0])) m |= 1u;
+            if (j4.y >= 0 && may_touch(xi, xj[1])) m |= 2u;
+            if (j4.z >= 0 && may_touch(xi, xj[2])) m |= 4u;
+            if (j4.w >= 0 && may_touch(xi, xj[3])) m |= 8u;
+            while (m) {
+                const int u = __ffs(m) - 1;
+                m &= m - 1;
+                const int j = u < 2 ? (u == 0 ? j4.x : j4.y) : (u == 2 ? j4.z : j4.w);
+                if (add_contact<kFric>(d, star, spin, xi, vi, i, off + e0 + u, j, X[j], F, T))
+                    in |= 1u << u;
+            }
         }
         if (kFric) {
             const unsigned there = (j4.x >= 0 ? 1u : 0u) | (j4.y >= 0 ? 2u : 0u) |
@@ -415,7 +433,7 @@ __device__ __forceinline__ int wall_scene(const DemDev &d, int i)
 // (d.omega, d.alpha).  rows: the rows may be read (contacts on, store not failed:
 // after LVB_EOVERFLOW the row offsets no longer fit the store).  The row
 // bounds and the scene are loaded with the particle's own state.
-template <bool kFric>
+template <bool kFric, bool kMany>
 __device__ __forceinline__ void forces_body(const DemDev &d, int i, const float4 *vin,
                                             const float4 *ain, const float4 *win,
                                             const float4 *alin)
@@ -429,7 +447,7 @@ __device__ __forceinline__ void forces_body(const DemDev &d, int i, const float4
     if (!d.contacts_on || (d.rows.cnt->err & DERR_STORE)) len = 0;
     const StoredStar star{d.vstar}, spin{d.wstar};
     float F[3] = {0.f, 0.f, 0.f}, T[3] = {0.f, 0.f, 0.f};
-    row_forces<kFric>(d, d.pos, star, spin, xi, vi, i, off, len, F, T);
+    row_forces<kFric, kMany>(d, d.pos, star, spin, xi, vi, i, off, len, F, T);
     wall_forces(d, xi, vi, sc_i, F);
     d.acc[i] = finish_velocity(d, F, vi.w, a, v);
     d.vel[i] = v;
@@ -452,7 +470,7 @@ k_forces(DemDev d)
     const int i = blockIdx.x * kThreads + threadIdx.x;
     if (i == 0) atomicAdd(d.rows.kernels, 1ULL);
     dtr_enter(d, TR_FORCES);
-    if (i < d.n) forces_body<kFric>(d, i, d.vel, d.acc, d.omega, d.alpha);
+    if (i < d.n) forces_body<kFric, false>(d, i, d.vel, d.acc, d.omega, d.alpha);
     dtr_exit(d, TR_FORCES);
 }
 
@@ -511,7 +529,7 @@ __device__ __forceinline__ void advance_pass(const DevState &s, const DemDev &d,
                 if (len > 0) {
                     const DerivedStar star{b.v[bv], b.a[bv], d.dt},
                         spin{b.w[bv], b.al[bv], d.dt};
-                    row_forces<kFric>(d, b.x[bx], star, spin, x, vi, i, off, len, F, Tq);
+                    row_forces<kFric, false>(d, b.x[bx], star, spin, x, vi, i, off, len, F, Tq);
                 }
                 wall_forces(d, x, vi, sc, F);
                 a = finish_velocity(d, F, vi.w, a, v);
@@ -562,6 +580,14 @@ __device__ __forceinline__ void advance_pass(const DevState &s, const DemDev &d,
 // straight to it), so the block barrier that follows the filling publishes it.
 static __shared__ DevState s_state;
 
+__device__ __forceinline__ void copy_state(const DevState &s)
+{
+    static_assert(sizeof(DevState) % 4 == 0, "copied in words");
+    for (int t = threadIdx.x; t < (int)(sizeof(DevState) / 4); t += blockDim.x)
+        reinterpret_cast<unsigned *>(&s_state)[t] = reinterpret_cast<const unsigned *>(&s)[t];
+    __syncthreads();
+}
+
 template <bool kPartial>
 static __device__ __noinline__ bool rest_of_step(const lvb_mlp_weights *w_sh, const float4 *pos,
                                                  const float4 *vel, const float4 *acc, bool inc,
@@ -596,10 +622,7 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
     const bool net = kPartial && s.skin_kind == LVB_SKIN_LEARNED;
     if (net) weights_copy_async(&w_sh, s.mlp);
     step_kernel_begin();
-    static_assert(sizeof(DevState) % 4 == 0, "copied in words");
-    for (int t = threadIdx.x; t < (int)(sizeof(DevState) / 4); t += blockDim.x)
-        reinterpret_cast<unsigned *>(&s_state)[t] = reinterpret_cast<const unsigned *>(&s)[t];
-    __syncthreads();   // s_state
+    copy_state(s);
     if (step_lead()) atomicAdd(&c->kernels, 1ULL);
     // v* of everyone at every step where the trigger may update anyone
     const bool star_always = !kPartial || s.early_beta < 1.0f;
@@ -628,11 +651,81 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
     flush_work(s);
     const unsigned long long t3 = (s.trace && step_lead()) ? global_ns() : 0ULL;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.n; i += gridDim.x * blockDim.x)
-        forces_body<kFric>(d, i, b.v[bv], b.a[bv], b.w[bv], b.al[bv]);
+        forces_body<kFric, false>(d, i, b.v[bv], b.a[bv], b.w[bv], b.al[bv]);
     if (s.trace) {
         if (!grid_barrier(s)) return;
         if (step_lead()) trace_add(c, TR_TAIL, t3, global_ns());
     }
+}
+
+// The same steps with the forces apart, for particles with many contacts: the
+// half-step and check, the rest of the step, the forces, a grid barrier; the
+// state in place, in d.pos, d.vel, d.acc.  A joined pass gathers v and a of a
+// partner in contact (w and al), these forces the stored v* (w*), and the gathers
+// bound a dense bed.  1M packed spheres in no order with 0.9, 1.5, 2.2 and 3.7
+// contacts each, us a step: joined 77, 86, 92 and 100, apart 78, 79, 76 and 78 (with
+// friction, 0.8, 1.2, 2.0 and 4.1 contacts: 163, 194, 240, 291 and 181, 194, 195, 210;
+// in the order of their places: 61, 67, 70, 72 and 75, 76, 74, 74).
+template <bool kFric, bool kPartial>
+__global__ void __launch_bounds__(kStepMaxThreads, 1)
+k_advance_apart(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
+                const __grid_constant__ DemBuffers b, int steps)
+{
+    DevCounters *c = s.cnt;
+    const unsigned err0 = c->err;
+    if (err0 & DERR_SYNC) return;
+    const unsigned done = (unsigned)c->steps;
+    __shared__ __align__(16) lvb_mlp_weights w_sh;
+    if (kPartial && s.skin_kind == LVB_SKIN_LEARNED) weights_copy_async(&w_sh, s.mlp);
+    step_kernel_begin();
+    copy_state(s);
+    if (step_lead()) atomicAdd(&c->kernels, 1ULL);
+    for (int k = 1; k <= steps; ++k) {
+        const unsigned long long t0 = (s.trace && step_lead()) ? global_ns() : 0ULL;
+        const unsigned err = k == 1 ? err0 : *(volatile unsigned *)&c->err;
+        const bool inc = kPartial && !(err & DERR_STORE);
+        const int step = next_step(done + k - 1), slot = step_slot(step);
+        grid_barrier_begin(slot);
+        advance_pass<kFric, false>(s, d, b, 0, 0, 0, false, true, inc, step, &c->nF_acc[slot]);
+        weights_copy_wait();
+        if (!rest_of_step<kPartial>(&w_sh, d.pos, d.vstar, d.acc, inc, step, slot, t0)) return;
+        const unsigned long long t3 = (s.trace && step_lead()) ? global_ns() : 0ULL;
+        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < d.n; i += gridDim.x * blockDim.x)
+            forces_body<kFric, true>(d, i, d.vel, d.acc, d.omega, d.alpha);
+        if (k < steps || s.trace) {   // the next half-step moves what others still read
+            if (!grid_barrier(s)) return;
+            if (s.trace && step_lead()) trace_add(c, TR_TAIL, t3, global_ns());
+        }
+    }
+    flush_work(s);
+}
+
+// The contacts of a sample of the particles, 32 to a warp from places spread over the
+// arrays, for the choice between the two: contacts in the upper half of *out
+// (host memory), particles in the lower.  One block.
+__global__ void __launch_bounds__(1024)
+k_sample(DemDev d, unsigned long long *out)
+{
+    __shared__ unsigned long long sum;
+    if (threadIdx.x == 0) {
+        sum = 0;
+        atomicAdd(d.rows.kernels, 1ULL);
+    }
+    __syncthreads();
+    const int warps = blockDim.x >> 5, chunks = (d.n + 31) / 32, q = threadIdx.x >> 5;
+    const int i = (int)((long long)q * chunks / min(warps, chunks)) * 32 + (threadIdx.x & 31);
+    if (q < chunks && i < d.n && !(d.rows.cnt->err & DERR_STORE)) {
+        const float4 xi = d.pos[i];
+        const int off = d.rows.row_off[i], len = min(d.rows.row_len[i], d.rows.row_cap[i]);
+        unsigned long long n = 0;
+        for (int e = 0; e < len; ++e) {
+            const int j = d.rows.col[off + e];
+            n += j >= 0 && may_touch(xi, d.pos[j]);
+        }
+        atomicAdd(&sum, (n << 32) + 1);
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) *(volatile unsigned long long *)out = sum;
 }
 
 // The contacts of the current state, each pair once (i < j from row i),
@@ -737,9 +830,13 @@ struct dem_ctx {
     dem_params prm{};
     lvb_ctx *bp = nullptr;
     cudaStream_t stream = nullptr;
-    int advance_blocks = 0;      // launch shape of k_advance, worked out for
-    int advance_threads = 0;     // the broad phase's step_version shape_of
-    int shape_of = -1;
+    int advance_blocks[2] = {0, 0};   // launch shapes of k_advance and k_advance_apart,
+    int advance_threads = 0;     // worked out for the broad phase's step_version
+    int shape_of = -1;           // shape_of
+    // the last sample of the contacts (k_sample; mapped host memory, null
+    // without contacts) and the steps enqueued since it was asked for
+    unsigned long long *sample = nullptr, *sample_d = nullptr;
+    int64_t since = 0;
 };
 
 namespace {
@@ -760,6 +857,7 @@ void dem_free(dem_ctx *c)
                       c->d.wstar, c->b.x[1], c->b.v[1], c->b.a[1], c->b.w[1], c->b.al[1]};
     for (float4 *p : ptrs)
         if (p) cudaFree(p);
+    if (c->sample) cudaFreeHost(c->sample);
 }
 
 // The driver's copy of the row-store addresses follows the broad phase's
@@ -788,32 +886,60 @@ int launch_phase(dem_ctx *c, int phase)
     return from_cuda(cudaGetLastError());
 }
 
-auto advance_kernel(const dem_ctx *c)
+auto advance_kernel(const dem_ctx *c, bool apart)
 {
-    if (step_state(c->bp).trigger == LVB_TRIGGER_PARTIAL)
-        return c->d.omega ? k_advance<true, true> : k_advance<false, true>;
+    const bool partial = step_state(c->bp).trigger == LVB_TRIGGER_PARTIAL;
+    if (apart) {
+        if (partial) return c->d.omega ? k_advance_apart<true, true> : k_advance_apart<false, true>;
+        return c->d.omega ? k_advance_apart<true, false> : k_advance_apart<false, false>;
+    }
+    if (partial) return c->d.omega ? k_advance<true, true> : k_advance<false, true>;
     return c->d.omega ? k_advance<true, false> : k_advance<false, false>;
 }
 
-// Launch shape of k_advance: the broad phase's block size, as many blocks as
-// are resident on the device at once, and no more than have work.
+// Asks for the contacts of a sample of the particles.  The answer is there when
+// the stream has come to it; until then the last one stands (both forms of the
+// steps give the same results).
+cudaError_t ask_sample(dem_ctx *c)
+{
+    if (!c->sample) return cudaSuccess;
+    c->since = 0;
+    k_sample<<<1, 1024, 0, c->stream>>>(c->d, c->sample_d);
+    return cudaGetLastError();
+}
+
+constexpr int64_t kSampleEvery = 500;   // steps (the sample takes as long as one or two)
+
+// Whether the particles have many contacts: one and a half each, in the sample.
+bool many_contacts(const dem_ctx *c)
+{
+    if (!c->sample) return false;
+    const unsigned long long v = *(volatile unsigned long long *)c->sample;
+    const unsigned contacts = (unsigned)(v >> 32), seen = (unsigned)v;
+    return seen > 0 && 2 * contacts >= 3 * seen;
+}
+
+// Launch shapes: the broad phase's block size, as many blocks as are resident on
+// the device at once, and no more than have work.
 int advance_shape(dem_ctx *c)
 {
     const int version = step_version(c->bp);
     if (c->shape_of == version) return LVB_OK;
-    int threads = 0, dev = 0, sms = 0, per_sm = 0;
+    int threads = 0, dev = 0, sms = 0;
     step_shape(c->bp, nullptr, &threads);
-    const void *fn = (const void *)advance_kernel(c);
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, threads, 0);
-    if (e != cudaSuccess) return from_cuda(e);
-    if (per_sm < 1) return LVB_EDEVICE;
     // a run of up to 2,048 particles stays on one block, whose barriers cost
     // next to nothing
     const int want = c->d.n <= 2 * threads ? 1 : (c->d.n + threads - 1) / threads;
-    c->advance_blocks = std::min(want, per_sm * sms);
+    for (int apart = 0; apart < 2 && e == cudaSuccess; ++apart) {
+        int per_sm = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+            &per_sm, (const void *)advance_kernel(c, apart), threads, 0);
+        if (e == cudaSuccess && per_sm < 1) return LVB_EDEVICE;
+        c->advance_blocks[apart] = std::min(want, per_sm * sms);
+    }
+    if (e != cudaSuccess) return from_cuda(e);
     c->advance_threads = threads;
     c->shape_of = version;
     return LVB_OK;
@@ -827,8 +953,14 @@ int launch_advance(dem_ctx *c, int steps)
     rc = advance_shape(c);
     if (rc) return rc;
     refresh(c);
-    const dim3 grid(c->advance_blocks), block(c->advance_threads);
-    return from_cuda(launch_coop(advance_kernel(c), grid, block, 0, c->stream,
+    if (c->since >= kSampleEvery) {
+        const cudaError_t e = ask_sample(c);
+        if (e != cudaSuccess) return from_cuda(e);
+    }
+    c->since += steps;
+    const bool apart = many_contacts(c);
+    const dim3 grid(c->advance_blocks[apart]), block(c->advance_threads);
+    return from_cuda(launch_coop(advance_kernel(c, apart), grid, block, 0, c->stream,
                                  step_state(c->bp), c->d, c->b, steps));
 }
 
@@ -891,6 +1023,14 @@ static int dem_init_impl(dem_ctx **out, int32_t n_scenes, const int64_t *offsets
         if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.w[1], sizeof(float4) * n);
         if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.al[1], sizeof(float4) * n);
     }
+    if (d.contacts_on) {
+        if (e == cudaSuccess)
+            e = cudaHostAlloc((void **)&c->sample, sizeof(*c->sample), cudaHostAllocMapped);
+        if (e == cudaSuccess) {
+            *c->sample = 0;
+            e = cudaHostGetDevicePointer((void **)&c->sample_d, c->sample, 0);
+        }
+    }
     if (e != cudaSuccess) {
         dem_free(c);
         delete c;
@@ -931,6 +1071,7 @@ static int dem_init_impl(dem_ctx **out, int32_t n_scenes, const int64_t *offsets
     d0.omega = d0.alpha = d0.wstar = nullptr;
     k_forces<false><<<grid_n(d.n), kThreads, 0, c->stream>>>(d0);
     e = cudaGetLastError();
+    if (e == cudaSuccess) e = ask_sample(c);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) {
         dem_free(c);
@@ -1095,6 +1236,10 @@ int dem_set_state(dem_ctx *c, const float *pos_r, const float *vel, const float 
         e = cudaGetLastError();
     }
     if (e == cudaSuccess && acc) e = cudaMemcpyAsync(c->d.acc, acc, b, cudaMemcpyDefault, c->stream);
+    if (e == cudaSuccess && pos_r) {
+        refresh(c);
+        e = ask_sample(c);
+    }
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
     return from_cuda(e);
 }
