@@ -113,9 +113,8 @@ int dem_batch_init(dem_ctx **out, int32_t n_scenes, const int64_t *offsets,
 #define DEM_GRAPH_STEPS 100
 
 /* dem_advance -- enqueue `steps` full steps (no synchronisation), up to
- * DEM_GRAPH_STEPS of them to a cooperative launch (one to a launch with
- * specular walls and contacts together).  Between launches the host grows a
- * store that asked to grow. */
+ * DEM_GRAPH_STEPS of them to a cooperative launch.  Between launches the host
+ * grows a store that asked to grow. */
 int dem_advance(dem_ctx *ctx, int64_t steps);
 
 /* dem_phase -- enqueue one phase (DEM_PHASE_*) of a step; a step is the

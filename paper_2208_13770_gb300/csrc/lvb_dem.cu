@@ -658,10 +658,11 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
     }
 }
 
-// The same steps with the forces apart, for particles with many contacts: the
-// half-step and check, the rest of the step, the forces, a grid barrier; the
-// state in place, in d.pos, d.vel, d.acc.  A joined pass gathers v and a of a
-// partner in contact (w and al), these forces the stored v* (w*), and the gathers
+// The same steps with the forces apart, for particles with many contacts and for
+// specular walls with contacts: the half-step and check, the rest of the step, the
+// forces, a grid barrier; the state in place, in d.pos, d.vel, d.acc.  A joined
+// pass gathers v and a of a partner in contact (w and al), these forces the stored
+// v* (w*), and the gathers
 // bound a dense bed.  1M packed spheres in no order with 0.9, 1.5, 2.2 and 3.7
 // contacts each, us a step: joined 77, 86, 92 and 100, apart 78, 79, 76 and 78 (with
 // friction, 0.8, 1.2, 2.0 and 4.1 contacts: 163, 194, 240, 291 and 181, 194, 195, 210;
@@ -958,7 +959,10 @@ int launch_advance(dem_ctx *c, int steps)
         if (e != cudaSuccess) return from_cuda(e);
     }
     c->since += steps;
-    const bool apart = many_contacts(c);
+    // mirrored velocities cannot be worked out again from v and a, as a joined
+    // pass does for a contact's partner
+    const bool mirrored = c->d.wall_kind == DEM_WALL_SPECULAR && c->d.contacts_on;
+    const bool apart = mirrored || many_contacts(c);
     const dim3 grid(c->advance_blocks[apart]), block(c->advance_threads);
     return from_cuda(launch_coop(advance_kernel(c, apart), grid, block, 0, c->stream,
                                  step_state(c->bp), c->d, c->b, steps));
@@ -1111,13 +1115,8 @@ int dem_advance(dem_ctx *c, int64_t steps)
 {
     if (!c || steps < 0) return LVB_EINVAL;
     cudaGetLastError();   // clear a stale error of an unrelated earlier call
-    // mirrored velocities cannot be worked out again from v and a, as a
-    // pass over several steps does for a contact's partner: with specular
-    // walls and contacts every step is a launch of its own
-    const bool single = c->d.wall_kind == DEM_WALL_SPECULAR && c->d.contacts_on;
-    const int64_t most = single ? 1 : DEM_GRAPH_STEPS;
     for (int64_t done = 0; done < steps;) {
-        const int64_t m = std::min(most, steps - done);
+        const int64_t m = std::min<int64_t>(DEM_GRAPH_STEPS, steps - done);
         const int rc = launch_advance(c, (int)m);
         if (rc) return rc;
         done += m;

@@ -124,6 +124,23 @@ def test_batch_of_squares(mu):
     b.close()
 
 
+@pytest.mark.parametrize("mu", [0.0, 0.5])
+@pytest.mark.parametrize("n,apart", [(24, 0.0), (2049, 0.0), (9000, 0.0), (2049, 3e-4)])
+def test_specular_walls_with_contacts(n, apart, mu):
+    # mirrored at the floor within the run, with many contacts and with few
+    lvb = _lvb()
+    a, b = [lvb.DEM(squares(n, mu, wall="specular", apart=apart)) for _ in range(2)]
+    down = (a.state()[1][:, 2] < -2.0).sum()
+    run((a, b), (3, 1, 97))
+    equal(lvb, a, b)
+    assert (a.state()[1][:, 2] < -2.0).sum() < down        # mirrored
+    k = a.lvb.stats()["kernels_executed"]
+    a.advance(100)
+    assert a.lvb.stats()["kernels_executed"] - k <= 4      # not a launch for every step
+    a.close()
+    b.close()
+
+
 @pytest.mark.parametrize("n", [700, 3000, 160_000])
 @pytest.mark.parametrize("calls", [(1, 2), (40, 61)])
 def test_packed_spheres_in_one_context(n, calls):
