@@ -113,8 +113,15 @@ int dem_batch_init(dem_ctx **out, int32_t n_scenes, const int64_t *offsets,
 #define DEM_GRAPH_STEPS 100
 
 /* dem_advance -- enqueue `steps` full steps (no synchronisation), up to
- * DEM_GRAPH_STEPS of them to a cooperative launch.  Between launches the host
- * grows a store that asked to grow. */
+ * DEM_GRAPH_STEPS of them to a cooperative launch.  A launch holds every SM
+ * until its steps are done (18 ms for 100 steps of 6.2M particles), and work on
+ * other streams waits for it; a program that wants to share the device sooner
+ * passes fewer steps at a time.  Between launches the host grows a store that
+ * asked to grow.
+ * The first call of more than one step allocates 48 bytes a particle (80 with
+ * friction) for a second copy of the state; where they are not to be had, and
+ * with specular walls and contacts together or many contacts a particle, the
+ * steps run in place.  The results are the same. */
 int dem_advance(dem_ctx *ctx, int64_t steps);
 
 /* dem_phase -- enqueue one phase (DEM_PHASE_*) of a step; a step is the

@@ -48,7 +48,8 @@ struct DemDev {
 
 // The two buffers of x, v, a (and, with friction, w, al) of k_advance, whose
 // steps read their partners' state in one and write their own in the
-// other; the first of each is the driver's own array.
+// other; the first of each is the driver's own array, the second are parts of one
+// allocation (b.x[1]), made when a launch first needs them.
 struct DemBuffers {
     float4 *x[2], *v[2], *a[2], *w[2], *al[2];
 };
@@ -855,7 +856,7 @@ void dem_free(dem_ctx *c)
 {
     if (c->bp) lvb_destroy(c->bp);
     float4 *ptrs[] = {c->d.pos, c->d.vel, c->d.acc, c->d.vstar, c->d.omega, c->d.alpha,
-                      c->d.wstar, c->b.x[1], c->b.v[1], c->b.a[1], c->b.w[1], c->b.al[1]};
+                      c->d.wstar, c->b.x[1]};
     for (float4 *p : ptrs)
         if (p) cudaFree(p);
     if (c->sample) cudaFreeHost(c->sample);
@@ -920,6 +921,34 @@ bool many_contacts(const dem_ctx *c)
     return seen > 0 && 2 * contacts >= 3 * seen;
 }
 
+// The second buffers of joined passes, 48 bytes a particle (80 with friction):
+// allocated when a launch first needs them, so that programs that never do keep
+// the memory.  Allowed while a stream is being captured.  False: there is not
+// enough memory (the form with the forces apart needs none).
+bool second_buffers(dem_ctx *c)
+{
+    if (c->b.x[1]) return true;
+    const size_t each = ((size_t)c->d.n + 15) / 16 * 16;   // on 256 bytes
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    float4 *p = nullptr;
+    const cudaError_t e =
+        cudaMalloc((void **)&p, sizeof(float4) * each * (c->d.omega ? 5 : 3));
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        cudaGetLastError();   // not this call's failure
+        return false;
+    }
+    c->b.x[1] = p;
+    c->b.v[1] = p + each;
+    c->b.a[1] = p + 2 * each;
+    if (c->d.omega) {
+        c->b.w[1] = p + 3 * each;
+        c->b.al[1] = p + 4 * each;
+    }
+    return true;
+}
+
 // Launch shapes: the broad phase's block size, as many blocks as are resident on
 // the device at once, and no more than have work.
 int advance_shape(dem_ctx *c)
@@ -962,7 +991,7 @@ int launch_advance(dem_ctx *c, int steps)
     // mirrored velocities cannot be worked out again from v and a, as a joined
     // pass does for a contact's partner
     const bool mirrored = c->d.wall_kind == DEM_WALL_SPECULAR && c->d.contacts_on;
-    const bool apart = mirrored || many_contacts(c);
+    const bool apart = mirrored || many_contacts(c) || (steps > 1 && !second_buffers(c));
     const dim3 grid(c->advance_blocks[apart]), block(c->advance_threads);
     return from_cuda(launch_coop(advance_kernel(c, apart), grid, block, 0, c->stream,
                                  step_state(c->bp), c->d, c->b, steps));
@@ -1017,15 +1046,10 @@ static int dem_init_impl(dem_ctx **out, int32_t n_scenes, const int64_t *offsets
     if (e == cudaSuccess) e = cudaMalloc((void **)&d.vel, sizeof(float4) * n);
     if (e == cudaSuccess) e = cudaMalloc((void **)&d.acc, sizeof(float4) * n);
     if (e == cudaSuccess) e = cudaMalloc((void **)&d.vstar, sizeof(float4) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.x[1], sizeof(float4) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.v[1], sizeof(float4) * n);
-    if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.a[1], sizeof(float4) * n);
     if (prm->mu > 0.0f) {
         if (e == cudaSuccess) e = cudaMalloc((void **)&d.omega, sizeof(float4) * n);
         if (e == cudaSuccess) e = cudaMalloc((void **)&d.alpha, sizeof(float4) * n);
         if (e == cudaSuccess) e = cudaMalloc((void **)&d.wstar, sizeof(float4) * n);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.w[1], sizeof(float4) * n);
-        if (e == cudaSuccess) e = cudaMalloc((void **)&c->b.al[1], sizeof(float4) * n);
     }
     if (d.contacts_on) {
         if (e == cudaSuccess)
