@@ -128,12 +128,28 @@ int lvb_mlp_grad(const float *samples, int64_t n, const float *params, const flo
  *   y_range     : host out, {y_lo, y_hi} from the labels' mean m and
  *                 standard deviation sd: y_lo = m / 16, y_hi = m + 4 sd.
  *   losses      : host out, mean loss of every epoch (epochs entries).
+ * Batches of up to 4,096 samples whose blocks (64 samples each) the device
+ * holds at once take one launch an epoch, others one for each batch and step.
  * Synchronises.  Errors: EINVAL, ENOMEM, EDEVICE, ETIMEOUT (the blocks of an
- * epoch's launch waited too long for one another).
+ * epoch's launch waited too long for one another; params unchanged).
  */
 int lvb_mlp_train(const float *samples, int64_t n, int32_t epochs, int32_t batch, float lr,
                   uint64_t seed, int32_t loss_kind, float *params, float *mu, float *isd,
                   float *y_range, float *losses, void *stream);
+
+/*
+ * lvb_mlp_train_limits -- lvb_mlp_train with limits on an epoch's launch: a hook
+ * for tests of what a smaller device or a stall would bring (the results are
+ * the same).
+ *   blocks_max : batches of more blocks than this take a launch each.
+ *   extra      : 1: every wait is for one arrival more than there are blocks, so
+ *                the first one runs out (ETIMEOUT); 0: normal.
+ *   spins      : polls before a wait gives up, 1 .. 2^22.
+ */
+int lvb_mlp_train_limits(const float *samples, int64_t n, int32_t epochs, int32_t batch, float lr,
+                         uint64_t seed, int32_t loss_kind, float *params, float *mu, float *isd,
+                         float *y_range, float *losses, void *stream, int32_t blocks_max,
+                         int32_t extra, int32_t spins);
 
 /*
  * lvb_mlp_travel_labels -- rebuild-log samples turned into training samples

@@ -393,7 +393,7 @@ __global__ void k_adam(float *p, const float *part, int nb, float *m, float *v, 
 // 10.8 us for 512 samples, against 37 us with a launch for each batch (one thread to a
 // sample) and one for each step.
 constexpr int kMaxTeam = 64;             // blocks of an epoch's launch
-constexpr unsigned kEpochSpins = 1u << 22;
+constexpr int kEpochSpins = 1 << 22;      // polls before a barrier gives up
 
 struct EpochArgs {
     const float *samples;
@@ -409,6 +409,7 @@ struct EpochArgs {
     float rel_floor;
     unsigned long long *arrived;         // grid barrier, zero at the start
     unsigned *failed;
+    unsigned extra, spins;               // arrivals waited for beyond the blocks', polls
 };
 
 struct EpochShared {
@@ -463,9 +464,10 @@ k_mlp_epoch(EpochArgs a)
             next = value(first + a.batch);
         }
         __syncthreads();
-        if (gridDim.x > 1) {
+        if (gridDim.x > 1 || a.extra) {
             if (t == 0) {
-                const unsigned long long need = (unsigned long long)(step + 1) * gridDim.x;
+                const unsigned long long need =
+                    (unsigned long long)(step + 1) * gridDim.x + a.extra;
                 asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(a.arrived), "l"(1ULL)
                              : "memory");
                 unsigned long long got = 0;
@@ -473,7 +475,7 @@ k_mlp_epoch(EpochArgs a)
                 do {
                     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];"
                                  : "=l"(got) : "l"(a.arrived) : "memory");
-                } while (got < need && ++it <= kEpochSpins);
+                } while (got < need && ++it <= a.spins);
                 if (got < need) atomicOr(a.failed, 1u);
                 s.ok = got >= need;
             }
@@ -558,6 +560,18 @@ int launch_batch(const float *samples, const int *order, int64_t first, int64_t 
     const int64_t blocks = (count + kTB - 1) / kTB;
     k_mlp_batch<<<(unsigned)blocks, kMlpThreads, sizeof(MlpTile), st>>>(a);
     return (int)blocks;
+}
+
+// Blocks of an epoch's launch that are resident on the device at once.
+int epoch_blocks(cudaError_t *e)
+{
+    int dev = 0, sms = 0, per_sm = 0;
+    *e = cudaGetDevice(&dev);
+    if (*e == cudaSuccess) *e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (*e == cudaSuccess)
+        *e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_mlp_epoch, kMlpThreads,
+                                                           sizeof(EpochShared));
+    return per_sm * sms;
 }
 
 constexpr int64_t kGradChunk = 1024 * kTB;   // samples per pass of lvb_mlp_grad
@@ -659,12 +673,23 @@ int lvb_mlp_train(const float *samples, int64_t n, int32_t epochs, int32_t batch
                   uint64_t seed, int32_t loss_kind, float *params, float *mu, float *isd,
                   float *y_range, float *losses, void *stream)
 {
+    return lvb_mlp_train_limits(samples, n, epochs, batch, lr, seed, loss_kind, params, mu, isd,
+                                y_range, losses, stream, kMaxTeam, 0, kEpochSpins);
+}
+
+int lvb_mlp_train_limits(const float *samples, int64_t n, int32_t epochs, int32_t batch, float lr,
+                         uint64_t seed, int32_t loss_kind, float *params, float *mu, float *isd,
+                         float *y_range, float *losses, void *stream, int32_t blocks_max,
+                         int32_t extra, int32_t spins)
+{
     if (!samples || n < 1 || epochs < 1 || batch < 1 || !(lr > 0.0f) || !params || !mu || !isd ||
         !y_range)
         return LVB_EINVAL;
     if (loss_kind != LVB_MLP_LOSS_SQUARED && loss_kind != LVB_MLP_LOSS_RELATIVE)
         return LVB_EINVAL;
     if (n > INT32_MAX) return LVB_EINVAL;
+    if (blocks_max < 0 || extra < 0 || extra > 1 || spins < 1 || spins > kEpochSpins)
+        return LVB_EINVAL;
     cudaGetLastError();
     const cudaStream_t st = (cudaStream_t)stream;
     // feature normalisation from the samples (mean, 1/std), label range
@@ -697,13 +722,16 @@ int lvb_mlp_train(const float *samples, int64_t n, int32_t epochs, int32_t batch
     // relative error: labels below the output range's floor count as the floor
     const float rel_floor = loss_kind == LVB_MLP_LOSS_RELATIVE ? std::max(y_range[0], 1e-30f)
                                                                : 0.0f;
-    // batches of up to kMaxTeam blocks: an epoch to a launch; larger ones: a
-    // launch for each batch and for each Adam step
+    // batches of up to kMaxTeam blocks that the device holds at once: an epoch to
+    // a launch; larger ones: a launch for each batch and for each Adam step (the
+    // same sums and steps)
     const int64_t batches = (n + batch - 1) / batch;
     const int64_t blocks = (std::min<int64_t>(batch, n) + kTB - 1) / kTB;
-    const bool epoch_launch = blocks <= kMaxTeam;
     DevBuf dp, dmu, disd, dg, dm, dv, dl, dord, dc, dbar;
     e = allow_shared();
+    const int resident = e == cudaSuccess ? epoch_blocks(&e) : 0;
+    const bool epoch_launch =
+        blocks <= std::min(std::min(kMaxTeam, resident), (int)blocks_max);
     if (e == cudaSuccess) e = dnew<float>(dp, NP);
     if (e == cudaSuccess) e = dnew<float>(dmu, NI);
     if (e == cudaSuccess) e = dnew<float>(disd, NI);
@@ -759,6 +787,8 @@ int lvb_mlp_train(const float *samples, int64_t n, int32_t epochs, int32_t batch
             a.rel_floor = rel_floor;
             a.arrived = (unsigned long long *)dbar.p;
             a.failed = (unsigned *)((unsigned long long *)dbar.p + 1);
+            a.extra = (unsigned)extra;
+            a.spins = (unsigned)spins;
             e = launch_coop(k_mlp_epoch, dim3((unsigned)blocks), dim3(kMlpThreads),
                             sizeof(EpochShared), st, a);
         } else {

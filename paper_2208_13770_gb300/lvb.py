@@ -106,6 +106,9 @@ _SIGS = {
                       _p], ctypes.c_int),
     "lvb_mlp_train": ([_p, _i64, ctypes.c_int32, ctypes.c_int32, ctypes.c_float, ctypes.c_uint64,
                        ctypes.c_int32, _p, _p, _p, _p, _p, _p], ctypes.c_int),
+    "lvb_mlp_train_limits": ([_p, _i64, ctypes.c_int32, ctypes.c_int32, ctypes.c_float,
+                              ctypes.c_uint64, ctypes.c_int32, _p, _p, _p, _p, _p, _p,
+                              ctypes.c_int32, ctypes.c_int32, ctypes.c_int32], ctypes.c_int),
     "lvb_mlp_travel_labels": ([_p, _i64, ctypes.c_int32, ctypes.c_float, ctypes.c_float, _p,
                                _pi64, _p], ctypes.c_int),
     "lvb_log_enable": ([_p, ctypes.c_int32, _i64], ctypes.c_int),
@@ -351,6 +354,13 @@ def lvb_mlp_train(samples, n, epochs, batch, lr, seed, loss_kind, params, mu, is
                   losses, stream=None):
     return _lib.lvb_mlp_train(samples, int(n), int(epochs), int(batch), float(lr), int(seed),
                               int(loss_kind), params, mu, isd, y_range, losses, stream)
+
+
+def lvb_mlp_train_limits(samples, n, epochs, batch, lr, seed, loss_kind, params, mu, isd, y_range,
+                         losses, blocks_max, extra, spins, stream=None):
+    return _lib.lvb_mlp_train_limits(samples, int(n), int(epochs), int(batch), float(lr), int(seed),
+                                     int(loss_kind), params, mu, isd, y_range, losses, stream,
+                                     int(blocks_max), int(extra), int(spins))
 
 
 def lvb_mlp_travel_labels(samples, n, horizon, margin, clip_q, out, n_out, stream=None):
