@@ -18,6 +18,7 @@
 #include <cmath>
 #include <cstddef>
 #include <cstring>
+#include <new>
 #include <random>
 #include <vector>
 
@@ -748,11 +749,18 @@ int lvb_mlp_train_limits(const float *samples, int64_t n, int32_t epochs, int32_
     if (e == cudaSuccess) e = cudaMemsetAsync(dm.p, 0, NP * 4, st);
     if (e == cudaSuccess) e = cudaMemsetAsync(dv.p, 0, NP * 4, st);
     if (e != cudaSuccess) return from_cuda(e);
-    std::vector<int> order((size_t)n), later;
+    std::vector<int> order, later;   // this epoch's order and the next one's
+    std::vector<float> c12;
+    try {
+        order.resize((size_t)n);
+        if (epochs > 1) later.resize((size_t)n);
+        if (epoch_launch) c12.resize((size_t)batches * 2);
+    } catch (const std::bad_alloc &) {
+        return LVB_ENOMEM;
+    }
     for (int64_t i = 0; i < n; ++i) order[(size_t)i] = (int)i;
     std::mt19937_64 rng(seed);
     const AdamStep ad{lr, 0.9f, 0.999f, 1e-8f};
-    std::vector<float> c12((size_t)(epoch_launch ? batches * 2 : 0));
     int64_t t = 0;
     std::shuffle(order.begin(), order.end(), rng);
     for (int ep = 0; ep < epochs; ++ep) {
