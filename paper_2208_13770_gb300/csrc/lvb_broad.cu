@@ -197,7 +197,7 @@ struct ScanArgs {
     const int *len;      // n sizes (before the transform)
     int *off;            // n (+1 if total_slot) offsets out
     int *cap;            // optional: transformed sizes out
-    int slack;           // 1: size = row_capacity(len); 0: size = len
+    int slack;           // 1: size = row_capacity(len), 2: slim; 0: size = len
     int n;
     long long *blk;      // ceil(n / kScanBlock) partials
     long long limit;     // total must not exceed this (else DERR_STORE)
@@ -208,7 +208,7 @@ __device__ __forceinline__ int scan_size(const ScanArgs &a, int i)
 {
     if (i >= a.n) return 0;
     const int l = a.len[i];
-    return a.slack ? row_capacity(l) : l;
+    return a.slack ? row_capacity(l, a.slack == 2) : l;
 }
 
 __device__ long long block_excl_scan(long long v, long long *total)
@@ -823,7 +823,7 @@ ScanArgs layout_args(lvb_ctx *c)
     a.len = c->s.row_len;
     a.off = c->s.row_off;
     a.cap = c->s.row_cap;
-    a.slack = 1;
+    a.slack = c->s.slim ? 2 : 1;
     a.n = (int)c->n;
     a.blk = c->s.blk;
     a.limit = c->s.col_cap;
@@ -892,6 +892,26 @@ int read_occupancy(lvb_ctx *c, Occupancy *o)
     return LVB_OK;
 }
 
+// Lays the counted rows out, whatever the store; *need: the entries they take.
+// Offsets are 32 bits: rows that would not fit with their usual slack get less.
+// Waits for the stream.
+int lay_out(lvb_ctx *c, long long *need)
+{
+    const long long cap0 = c->s.col_cap;
+    int rc = LVB_OK;
+    for (int k = 0; k < 2; ++k) {
+        c->s.col_cap = 1LL << 62;
+        launch_layout_scan(c, GATE_ALWAYS);
+        rc = sync_counters(c);
+        c->s.col_cap = cap0;
+        if (rc) return rc;
+        *need = c->cnt_h->store_needed;
+        if (*need <= INT32_MAX || c->s.slim) break;
+        c->s.slim = 1;
+    }
+    return rc;
+}
+
 // Grows the row store and/or the cell slots when a kernel asked for it
 // (over 75% full), then rebuilds the cells and rows from the current
 // reference state -- the list is a function of that state alone, so the
@@ -930,13 +950,9 @@ int grow_if_asked(lvb_ctx *c)
     }
     // rows: count, then a store with room to grow, then fill
     k_rows<<<rows_grid(c), kThreads, 0, st>>>(s, GATE_ALWAYS, 0);
-    const long long cap0 = s.col_cap;
-    s.col_cap = 1LL << 62;
-    launch_layout_scan(c, GATE_ALWAYS);
-    int rc = sync_counters(c);
-    s.col_cap = cap0;
+    long long need = 0;
+    const int rc = lay_out(c, &need);
     if (rc) return rc;
-    const long long need = c->cnt_h->store_needed;
     bool grown = false;
     if (need * 5 > s.col_cap * 3) {   // over 60%: grow
         const long long cap = std::min<long long>(2 * need + 8 * c->n + 1024, INT32_MAX);
@@ -1350,12 +1366,9 @@ static int init_impl(lvb_ctx **out, int nscenes, const int64_t *offsets, int64_t
 
     // rows: count, lay out with slack, allocate the store, fill
     k_rows<<<rows_grid(c), kThreads, 0, st>>>(s, GATE_ALWAYS, 0);
-    s.col_cap = (1LL << 62);
-    c->s = s;
-    launch_layout_scan(c, GATE_ALWAYS);
-    rc = sync_counters(c);
+    long long needed = 0;
+    rc = lay_out(c, &needed);
     if (rc) return fail(rc);
-    const long long needed = c->cnt_h->store_needed;
     long long col_cap = std::max<long long>(2 * needed + 8 * n + 1024, 4096);
     if (col_cap > INT32_MAX) col_cap = INT32_MAX;
     if (needed > col_cap) return fail(LVB_ENOMEM);

@@ -251,12 +251,14 @@ __device__ __forceinline__ float mlp_skin(const lvb_mlp_weights *__restrict__ W,
 // for the row to grow by half, and by 8 however short it is, before the
 // store is re-laid out).  Every row's capacity, with slack or without, is a
 // multiple of four, so that every row starts on a 16-byte boundary and is
-// read four entries at a time (entries past the row's length hold -1).
+// read four entries at a time (entries past the row's length hold -1).  slim:
+// that multiple is the next lower one, for stores that would not fit 2^31
+// entries otherwise.
 __host__ __device__ __forceinline__ int row_tight(int len) { return (len + 3) & ~3; }
 
-__host__ __device__ __forceinline__ int row_capacity(int len)
+__host__ __device__ __forceinline__ int row_capacity(int len, bool slim)
 {
-    return row_tight(len + 8 + (len >> 1));
+    return (len + 8 + (len >> 1) + (slim ? 0 : 3)) & ~3;
 }
 
 }  // namespace lvb

@@ -72,6 +72,7 @@ struct DevState {
     // it are -1; row_len[i] > row_cap[i] means the row overflowed
     int *row_off, *row_len, *row_cap, *col;
     long long col_cap;
+    int slim;         // rows have the smaller slack (row_capacity)
     int *cell_cnt, *cell_id;
     float4 *cell_ref;
     DevCounters *cnt;
@@ -1614,7 +1615,7 @@ static __device__ long long layout_scan(const DevState &s, bool tight)
     const int hi = (int)min((long long)s.n, lo + per);
     long long sum = 0, tot;
     for (int i = lo + threadIdx.x; i < hi; i += blockDim.x)
-        sum += tight ? row_tight(s.row_len[i]) : row_capacity(s.row_len[i]);
+        sum += tight ? row_tight(s.row_len[i]) : row_capacity(s.row_len[i], s.slim);
     block_scan_any(sum, &tot);
     if (threadIdx.x == 0) s.blk[blockIdx.x] = tot;
     if (!grid_barrier(s)) return -1;
@@ -1638,7 +1639,7 @@ static __device__ long long layout_scan(const DevState &s, bool tight)
     for (int i0 = lo; i0 < hi; i0 += blockDim.x) {
         const int i = i0 + threadIdx.x;
         const int v =
-            i < hi ? (tight ? row_tight(s.row_len[i]) : row_capacity(s.row_len[i])) : 0;
+            i < hi ? (tight ? row_tight(s.row_len[i]) : row_capacity(s.row_len[i], s.slim)) : 0;
         const long long ex = block_scan_any(v, &tot);
         if (i < hi) {
             s.row_off[i] = (int)min(run + ex, (long long)INT32_MAX);
