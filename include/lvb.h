@@ -327,7 +327,7 @@ int lvb_step_host(lvb_ctx *ctx, const float *pos_r, const float *vel, const floa
  * invalid, as always): */
 #define LVB_OPT_GROW 10       /* 1 (default): the host grows the cell slots and
                                 the row store between steps when a kernel
-                                finds them over 75% / 60% full; 0: requests
+                                finds them over 75% / 67% full; 0: requests
                                 are ignored, so a cell that fills up reports
                                 LVB_EOVERFLOW */
 #define LVB_OPT_FORCE_RELAYOUT 14 /* 1: the next step that rebuilds rows

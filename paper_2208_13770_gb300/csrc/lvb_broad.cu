@@ -248,7 +248,18 @@ k_scan_reduce(ScanArgs a, DevState s, int gate)
     count_kernel(s);
     const int b = blockIdx.x;
     long long sum = 0;
-    for (int k = 0; k < kScanPer; ++k) sum += scan_size(a, b * kScanBlock + k * kThreads + threadIdx.x);
+    int pad = 0;
+    for (int k = 0; k < kScanPer; ++k) {
+        const int i = b * kScanBlock + k * kThreads + threadIdx.x, v = scan_size(a, i);
+        sum += v;
+        if (a.slack && i < a.n) pad += v - row_slack(a.len[i]);
+    }
+    if (a.slack) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) pad += __shfl_xor_sync(FULL, pad, o);
+        if ((threadIdx.x & 31) == 0 && pad)
+            atomicAdd((unsigned long long *)&s.cnt->store_padding, (unsigned long long)(long long)pad);
+    }
     long long tot;
     block_excl_scan(sum, &tot);
     if (threadIdx.x == 0) a.blk[b] = tot;
@@ -895,20 +906,25 @@ int read_occupancy(lvb_ctx *c, Occupancy *o)
     return LVB_OK;
 }
 
-// Lays the counted rows out, whatever the store; *need: the entries they take.
+// Lays the counted rows out, whatever the store; *need: the entries they take,
+// *alloc: the entries to allocate for them.
 // Offsets are 32 bits: rows that would not fit with their usual slack get less.
 // Waits for the stream.
-int lay_out(lvb_ctx *c, long long *need)
+int lay_out(lvb_ctx *c, long long *need, long long *alloc)
 {
     const long long cap0 = c->s.col_cap;
     int rc = LVB_OK;
     for (int k = 0; k < 2; ++k) {
+        const cudaError_t e = cudaMemsetAsync(&c->s.cnt->store_padding, 0, sizeof(long long),
+                                              c->stream);
+        if (e != cudaSuccess) return from_cuda(e);
         c->s.col_cap = 1LL << 62;
         launch_layout_scan(c, GATE_ALWAYS);
         rc = sync_counters(c);
         c->s.col_cap = cap0;
         if (rc) return rc;
         *need = c->cnt_h->store_needed;
+        *alloc = std::min<long long>(store_entries(*need, c->cnt_h->store_padding, c->n), INT32_MAX);
         if (*need <= INT32_MAX || c->s.slim) break;
         c->s.slim = 1;
     }
@@ -953,12 +969,11 @@ int grow_if_asked(lvb_ctx *c)
     }
     // rows: count, then a store with room to grow, then fill
     rows_kernel(c)<<<rows_grid(c), kThreads, 0, st>>>(s, GATE_ALWAYS, 0, 0);
-    long long need = 0;
-    const int rc = lay_out(c, &need);
+    long long need = 0, cap = 0;
+    const int rc = lay_out(c, &need, &cap);
     if (rc) return rc;
     bool grown = false;
-    if (need * 5 > s.col_cap * 3) {   // over 60%: grow
-        const long long cap = std::min<long long>(2 * need + 8 * c->n + 1024, INT32_MAX);
+    if (need * 3 > s.col_cap * 2) {   // over two thirds: grow
         if (need > cap) return LVB_ENOMEM;
         cudaFree(s.col);
         s.col = nullptr;
@@ -1369,11 +1384,10 @@ static int init_impl(lvb_ctx **out, int nscenes, const int64_t *offsets, int64_t
 
     // rows: count, lay out with slack, allocate the store, fill
     rows_kernel(c)<<<rows_grid(c), kThreads, 0, st>>>(s, GATE_ALWAYS, 0, 0);
-    long long needed = 0;
-    rc = lay_out(c, &needed);
+    long long needed = 0, col_cap = 0;
+    rc = lay_out(c, &needed, &col_cap);
     if (rc) return fail(rc);
-    long long col_cap = std::max<long long>(2 * needed + 8 * n + 1024, 4096);
-    if (col_cap > INT32_MAX) col_cap = INT32_MAX;
+    col_cap = std::max<long long>(col_cap, 4096);
     if (needed > col_cap) return fail(LVB_ENOMEM);
     e = dalloc(&s.col, col_cap);
     if (e != cudaSuccess) return fail(from_cuda(e));

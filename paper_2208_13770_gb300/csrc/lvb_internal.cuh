@@ -56,6 +56,8 @@ struct DevCounters {
     long long updated_total;
     long long relayouts;
     long long store_needed;  // entries the row store needed at the last layout
+    long long store_padding; // of those, what the host's last layout added to rows
+                             // to make their capacities multiples of four
     unsigned long long kernels;  // kernels of this library executed (device count)
     unsigned long long barriers; // grid barriers passed by step kernels
     long long ex_total;      // entries of the last export
@@ -255,10 +257,20 @@ __device__ __forceinline__ float mlp_skin(const lvb_mlp_weights *__restrict__ W,
 // that multiple is the next lower one, for stores that would not fit 2^31
 // entries otherwise.
 __host__ __device__ __forceinline__ int row_tight(int len) { return (len + 3) & ~3; }
+__host__ __device__ __forceinline__ int row_slack(int len) { return len + 8 + (len >> 1); }
 
 __host__ __device__ __forceinline__ int row_capacity(int len, bool slim)
 {
-    return (len + 8 + (len >> 1) + (slim ? 0 : 3)) & ~3;
+    return slim ? row_slack(len) & ~3 : row_tight(row_slack(len));
+}
+
+// Entries to allocate for rows that take `need` now, `padding` of them by the
+// rounding to multiples of four: twice the rows with their slack and room for
+// eight more each (the padding does not count, so the memory is what unrounded
+// rows would get; it is three entries a row at most).
+inline long long store_entries(long long need, long long padding, long long n)
+{
+    return 2 * (need - padding) + 8 * n + 1024;
 }
 
 }  // namespace lvb

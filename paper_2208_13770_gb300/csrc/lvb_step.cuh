@@ -1654,7 +1654,7 @@ static __device__ long long layout_scan(const DevState &s, bool tight)
 // from the (final) cells, offsets with slack, rows filled.  When the rows
 // with slack do not fit the store they are laid out tight (no slack; the
 // next edits re-lay out again) and, if even that does not fit, the store
-// has failed (DERR_STORE).  A layout above 60% of the store asks the host
+// has failed (DERR_STORE).  A layout above two thirds of the store asks the host
 // to grow it before the next step.  Returns false when the step must be
 // abandoned.
 static __device__ __noinline__ bool relayout_pass(const DevState &s)
@@ -1686,7 +1686,8 @@ static __device__ __noinline__ bool relayout_pass(const DevState &s)
         c->force_relayout = 0;
         c->relayouts += 1;
         c->store_needed = need;
-        if (need * 5 > s.col_cap * 3) {        // over 60% of the store: grow it
+        // (rows rounded to multiples of four; 60% before, of rows that were not)
+        if (need * 3 > s.col_cap * 2) {
             s.hflags->store_needed = need;
             s.hflags->grow_store = 1;
         }

@@ -34,3 +34,20 @@ def test_rows_get_less_slack_where_the_store_needs_it():
     st = ctx.stats()
     assert st["flagged_total"] == 1 and st["entries"] == 2 * (pairs - 1)
     ctx.close()
+
+
+@pytest.mark.parametrize("n", [1, 700, 30_000])
+def test_rounded_rows_take_no_more_memory(n):
+    # the store: twice the rows with a slack of half their length and eight, and
+    # room for eight more each, whatever the capacities are rounded to
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import numpy as np
+    from paper_2208_13770_gb300 import lvb, scenes
+    for s in (scenes.packed(n=n, seed=5), scenes.settling(n=n, seed=5, footprint=0.1)):
+        ctx = lvb.LVB(torch.from_numpy(s.pos).cuda(), s.lo, s.hi, lvb.LVB_SKIN_DIAMETER_FACTOR, 0.1,
+                      s.dt, lvb.LVB_TRIGGER_PARTIAL, s.cell_factor)
+        rows = np.diff(ctx.pairs_csr()[0]).astype(np.int64)
+        want = 2 * int((rows + 8 + rows // 2).sum()) + 8 * n + 1024
+        assert ctx.stats()["row_store_capacity"] == max(want, 4096)
+        ctx.close()
