@@ -34,7 +34,10 @@ constexpr int kStepMaxThreads = 1024;     // block size limit of k_step (one blo
 constexpr int kCheckUnroll = 2;           // chunks of 32 particles a warp of the step kernel
                                           // should find at least (sizes its grid)
 constexpr int kFlaggedDirectMax = 4096;   // default of DevState::direct_max
-constexpr int kDirectUnroll = 4;          // flagged reference states per lane in flight
+// flagged reference states per lane in flight (2,000 flagged of 200k: with 4, 6 and
+// 8 a step takes 63, 53 and 57 us, with history 77, 71 and 69; 60 of 6,000: 24.6,
+// 24.8 and 26.1)
+constexpr int kDirectUnroll = 6;
 constexpr unsigned kBarrierSpins = 1u << 22;   // ~1-3 s of polling (L2 round trips) before a barrier gives up
 
 // Written by kernels straight into mapped host memory: requests to grow a
@@ -827,7 +830,7 @@ __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int 
         if (kHist) take = take && !pair_hit(s.oref[k], s.pold[j]);
         append(take, j);
     };
-    flagged(jf0, rf0);
+    if (m_dir) flagged(jf0, rf0);
     // 2. stencil and 3. insertions
     // Candidates that pass the pair test are only noted at first (kDense: their
     // slots, else their ids) and taken up together, up to 32 at a time: what
