@@ -118,10 +118,11 @@ int dem_batch_init(dem_ctx **out, int32_t n_scenes, const int64_t *offsets,
  * other streams waits for it; a program that wants to share the device sooner
  * passes fewer steps at a time.  Between launches the host grows a store that
  * asked to grow.
- * The first call of more than one step allocates 48 bytes a particle (80 with
- * friction) for a second copy of the state; where they are not to be had, and
- * with specular walls and contacts together or many contacts a particle, the
- * steps run in place.  The results are the same. */
+ * Steps of one launch use a second copy of the state, 48 bytes a particle (80
+ * with friction).  dem_init allocates it if it is at most an eighth of the free
+ * memory, otherwise the first call of more than one step does; where it is not to
+ * be had, and with specular walls and contacts together or many contacts a
+ * particle, the steps run in place.  The results are the same. */
 int dem_advance(dem_ctx *ctx, int64_t steps);
 
 /* dem_phase -- enqueue one phase (DEM_PHASE_*) of a step; a step is the

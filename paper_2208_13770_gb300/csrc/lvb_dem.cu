@@ -49,7 +49,7 @@ struct DemDev {
 // The two buffers of x, v, a (and, with friction, w, al) of k_advance, whose
 // steps read their partners' state in one and write their own in the
 // other; the first of each is the driver's own array, the second are parts of one
-// allocation (b.x[1]), made when a launch first needs them.
+// allocation (b.x[1]): second_buffers.
 struct DemBuffers {
     float4 *x[2], *v[2], *a[2], *w[2], *al[2];
 };
@@ -921,19 +921,30 @@ bool many_contacts(const dem_ctx *c)
     return seen > 0 && 2 * contacts >= 3 * seen;
 }
 
-// The second buffers of joined passes, 48 bytes a particle (80 with friction):
-// allocated when a launch first needs them, so that programs that never do keep
-// the memory.  Allowed while a stream is being captured.  False: there is not
-// enough memory (the form with the forces apart needs none).
-bool second_buffers(dem_ctx *c)
+// Whether the steps keep their forces apart.  (Mirrored velocities cannot be worked
+// out again from v and a, as a joined pass does for a contact's partner.)
+bool keeps_apart(const dem_ctx *c)
+{
+    return (c->d.wall_kind == DEM_WALL_SPECULAR && c->d.contacts_on) || many_contacts(c);
+}
+
+// The second buffers of joined passes, 48 bytes a particle (80 with friction).
+// dem_init allocates them where they are a small part of the memory (spare: only
+// if they are at most an eighth of what is free), so that the first call need not;
+// otherwise a launch that needs them does, also while a stream is being captured,
+// and a program that never has one keeps the memory.  False: there is not enough
+// (the form with the forces apart needs none).
+bool second_buffers(dem_ctx *c, bool spare = false)
 {
     if (c->b.x[1]) return true;
     const size_t each = ((size_t)c->d.n + 15) / 16 * 16;   // on 256 bytes
+    const size_t bytes = sizeof(float4) * each * (c->d.omega ? 5 : 3);
+    size_t room = 0, all = 0;
+    if (spare && (cudaMemGetInfo(&room, &all) != cudaSuccess || bytes > room / 8)) return false;
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     cudaThreadExchangeStreamCaptureMode(&mode);
     float4 *p = nullptr;
-    const cudaError_t e =
-        cudaMalloc((void **)&p, sizeof(float4) * each * (c->d.omega ? 5 : 3));
+    const cudaError_t e = cudaMalloc((void **)&p, bytes);
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (e != cudaSuccess) {
         cudaGetLastError();   // not this call's failure
@@ -988,10 +999,7 @@ int launch_advance(dem_ctx *c, int steps)
         if (e != cudaSuccess) return from_cuda(e);
     }
     c->since += steps;
-    // mirrored velocities cannot be worked out again from v and a, as a joined
-    // pass does for a contact's partner
-    const bool mirrored = c->d.wall_kind == DEM_WALL_SPECULAR && c->d.contacts_on;
-    const bool apart = mirrored || many_contacts(c) || (steps > 1 && !second_buffers(c));
+    const bool apart = keeps_apart(c) || (steps > 1 && !second_buffers(c));
     const dim3 grid(c->advance_blocks[apart]), block(c->advance_threads);
     return from_cuda(launch_coop(advance_kernel(c, apart), grid, block, 0, c->stream,
                                  step_state(c->bp), c->d, c->b, steps));
@@ -1106,6 +1114,7 @@ static int dem_init_impl(dem_ctx **out, int32_t n_scenes, const int64_t *offsets
         delete c;
         return from_cuda(e);
     }
+    if (!keeps_apart(c)) second_buffers(c, true);
     *out = c;
     return LVB_OK;
 }

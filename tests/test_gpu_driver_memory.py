@@ -1,6 +1,7 @@
 """Device memory of the DEM driver: the second copy of the state, which joined
-steps go back and forth between, is allocated by the first call that needs it,
-also inside a capture."""
+steps go back and forth between, is allocated by dem_init where it is a small part
+of the free memory, else by the first call that needs it, also inside a capture;
+and without it the same steps run in place."""
 import numpy as np
 import pytest
 
@@ -23,28 +24,73 @@ def _gas(n):
     return s
 
 
-def test_phases_and_single_steps_take_no_second_copy():
+def _free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info()[0]
+
+
+@pytest.fixture(scope="module")
+def measured():
+    """(n, bytes of a context of n without its second copy, its state after 5 steps);
+    all kernels loaded."""
     lvb = _lvb()
-    small = lvb.DEM(_gas(3000))            # the kernels are loaded
-    for m in (1, 3):
-        small.advance(m)
-    small.step()
-    small.sync()
-    small.close()
-    n = 4_000_000
-    dem = lvb.DEM(_gas(n))
-
-    def taken(f):
-        torch.cuda.synchronize()
-        before = torch.cuda.mem_get_info()[0]
-        f()
+    packed = scenes.packed(n=700)
+    packed.wall = "specular"
+    for s in (packed, _gas(3000)):
+        dem = lvb.DEM(s)
+        dem.advance(1)
+        dem.advance(3)
+        dem.step()
         assert dem.sync() == lvb.LVB_OK
-        return before - torch.cuda.mem_get_info()[0]
+        dem.close()
+    n = 6_000_000
+    for _ in range(2):                     # the first fills the caching allocator
+        before = _free()
+        dem = lvb.DEM(_gas(n))
+        bytes_ = before - _free() - 48 * n
+        dem.advance(5)
+        state = dem.state()
+        dem.close()
+    return n, bytes_, state
 
-    assert taken(dem.step) < 8 << 20
-    assert taken(lambda: dem.advance(1)) < 8 << 20
-    assert 48 * n <= taken(lambda: dem.advance(2)) < 48 * n + (8 << 20)
-    assert taken(lambda: dem.advance(20)) < 8 << 20
+
+@pytest.mark.parametrize("copies", [6, 0.5])
+def test_second_copy_where_memory_is_short(measured, copies):
+    # so much is left after dem_init: six copies (not an eighth), half a copy (the
+    # steps run in place)
+    lvb = _lvb()
+    n, bytes_, state = measured
+    lvb.DEM(_gas(n)).close()               # (the caching allocator holds the inputs' memory)
+    filler = torch.empty(_free() - bytes_ - int(copies * 48 * n), dtype=torch.uint8, device="cuda")
+    dem = None
+    try:
+        dem = lvb.DEM(_gas(n))
+        left = _free()
+        assert abs(left - copies * 48 * n) < 64 << 20
+        dem.advance(1)
+        assert dem.sync() == lvb.LVB_OK
+        assert left - _free() < 4 << 20
+        dem.advance(4)
+        assert dem.sync() == lvb.LVB_OK
+        taken = left - _free()
+        assert (48 * n <= taken < 48 * n + (8 << 20)) if copies > 1 else taken < 4 << 20
+        for x, y in zip(dem.state(), state):
+            assert np.array_equal(x, y)
+    finally:
+        if dem is not None:
+            dem.close()
+        del filler
+        torch.cuda.empty_cache()
+
+
+def test_second_copy_where_memory_is_plenty(measured):
+    lvb = _lvb()
+    n, bytes_, _ = measured
+    lvb.DEM(_gas(n)).close()
+    before = _free()
+    dem = lvb.DEM(_gas(n))
+    taken = before - _free()
+    assert abs(taken - bytes_ - 48 * n) < 8 << 20
     dem.close()
 
 
