@@ -376,8 +376,10 @@ int lvb_step_host(lvb_ctx *ctx, const float *pos_r, const float *vel, const floa
 /* Phases of the step kernel: 0 check (with the flagged particles'
  * updates; inside dem_advance also the forces of the step before and the
  * position half-step), 1 rebuild passes, 2 re-layout, 3 tail (the forces of
- * the last step of a dem_advance launch); separate kernels: 4 DEM integrate, 5 DEM forces, 6 full-build
- * rows (init, store growth); inside the partial rebuild: 7 from the first
+ * the last step of a dem_advance launch; of every step where they are not
+ * joined with the next check); separate kernels: 4 DEM integrate, 5 DEM
+ * forces, 6 full-build rows (init, store growth); inside the partial rebuild:
+ * 7 from the first
  * work item's start to the last one's end (patches and moves), 8 the
  * longest single work item. */
 

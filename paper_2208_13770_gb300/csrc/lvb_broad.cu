@@ -1870,10 +1870,9 @@ DevState step_state(lvb_ctx *c)
     return c->s;
 }
 
-void step_shape(lvb_ctx *c, int *blocks, int *threads)
+int step_threads(const lvb_ctx *c)
 {
-    if (blocks) *blocks = c->step_blocks;
-    *threads = c->block_threads;
+    return c->block_threads;
 }
 
 cudaStream_t step_stream(lvb_ctx *c)

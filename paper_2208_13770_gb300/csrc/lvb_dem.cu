@@ -3,7 +3,8 @@
 // Per step: position half-step (x', v*), the broad-phase step at x'
 // (displacement check and partial rebuild), forces (narrow phase on the
 // list rows, linear spring-dashpot, walls, a', v').  dem_advance runs up to
-// DEM_GRAPH_STEPS steps as one cooperative launch (k_advance); dem_phase runs
+// DEM_GRAPH_STEPS steps as one cooperative launch (k_advance, or k_advance_apart
+// where the particles have many contacts); dem_phase runs
 // the three parts as separate launches (k_integrate, lvb_step, k_forces), with
 // identical results.  Forces are accumulated per row of the
 // symmetric list, so each pair is evaluated once from each side and no
@@ -966,8 +967,8 @@ int advance_shape(dem_ctx *c)
 {
     const int version = step_version(c->bp);
     if (c->shape_of == version) return LVB_OK;
-    int threads = 0, dev = 0, sms = 0;
-    step_shape(c->bp, nullptr, &threads);
+    const int threads = step_threads(c->bp);
+    int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // a run of up to 2,048 particles stays on one block, whose barriers cost

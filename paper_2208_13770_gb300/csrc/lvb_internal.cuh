@@ -282,8 +282,8 @@ namespace lvb {
 // integrate kernel and by the kernel that advances whole steps (identical
 // arithmetic either way: explicit roundings, no compiler-chosen fusion):
 //   x' = x + (v dt + a dt^2/2),  v* = v + a dt   (v*.w keeps 1/m)
-// with specular reflection at the scene box when `specular` (x mirrored, v
-// and v* negated per axis; returns true if v may have changed).
+// and, at specular walls, the reflection at the scene's box: x mirrored, v and v*
+// negated per axis.
 __device__ __forceinline__ float4 star_of(float4 v, float4 ac, float dt)
 {
     return make_float4(fmaf(ac.x, dt, v.x), fmaf(ac.y, dt, v.y), fmaf(ac.z, dt, v.z), v.w);
@@ -339,7 +339,7 @@ RowsView rows_view(lvb_ctx *c);
 // The device state a step kernel takes by value, and the launch shape of
 // the step kernel (blocks: all co-resident; threads per block).
 DevState step_state(lvb_ctx *c);
-void step_shape(lvb_ctx *c, int *blocks, int *threads);
+int step_threads(const lvb_ctx *c);
 cudaStream_t step_stream(lvb_ctx *c);
 // Waits for the context's stream and reads its counters back: the sticky device
 // error, and the counters through *host (valid until the next such call).

@@ -485,37 +485,6 @@ __device__ __forceinline__ void lane_remove(const DevState &s, int j, int i)
     }
 }
 
-// Adds partner i to unflagged row j (one lane): a -1 entry below row_len,
-// claimed with compare-and-swap, else the next slot at the end (also by
-// compare-and-swap: a slot past row_len holds -1 and another warp's search
-// may claim it first).  A full row raises *ovf (the re-layout rebuilds it).
-__device__ __forceinline__ void lane_insert(const DevState &s, int j, int i, int *ovf)
-{
-    const int off = s.row_off[j], cap = s.row_cap[j], len = min(s.row_len[j], cap);
-    for (int e = 0; e < len; e += 4) {
-        int v[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) v[u] = e + u < len ? s.col[off + e + u] : 0;
-#pragma unroll
-        for (int u = 0; u < 4; ++u)
-            if (v[u] < 0 && atomicCAS(&s.col[off + e + u], -1, i) == -1) {
-                if (s.hist) s.hist[off + e + u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                return;
-            }
-    }
-    for (int t = 0; t <= cap; ++t) {
-        const int p = atomicAdd(&s.row_len[j], 1);
-        if (p >= cap) {
-            atomicExch(ovf, 1);
-            return;
-        }
-        if (atomicCAS(&s.col[off + p], -1, i) == -1) {
-            if (s.hist) s.hist[off + p] = make_float4(0.f, 0.f, 0.f, 0.f);
-            return;
-        }
-    }
-}
-
 // Where a row lies: read ahead of an edit of it.
 struct RowSpan {
     int off, len, cap;
@@ -535,8 +504,11 @@ __device__ __forceinline__ RowSpan row_span(const DevState &s, int j)
 // One removal (partner i leaves row jr, which lies at r) and one insertion
 // (partner i joins row ji, which lies at q) by one lane, their loads
 // interleaved so that both edits take the latency of one: four entries of each
-// row at a time.  jr or ji < 0: no such edit.  Same rules as lane_remove and
-// lane_insert (the two rows differ: a removed pair is not a new one).
+// row at a time.  jr or ji < 0: no such edit (the two rows differ: a removed pair is
+// not a new one).  The removed entry becomes -1.  The new one takes a -1 entry
+// below row_len, claimed with compare-and-swap, else the next slot at the end,
+// also by compare-and-swap: a slot past row_len holds -1 and another warp's
+// search may claim it first.  A full row raises *ovf (the re-layout rebuilds it).
 __device__ __forceinline__ void lane_edit(const DevState &s, int jr, RowSpan r, int ji, RowSpan q,
                                           int i, int *ovf)
 {
