@@ -664,11 +664,13 @@ k_advance(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
 // specular walls with contacts: the half-step and check, the rest of the step, the
 // forces, a grid barrier; the state in place, in d.pos, d.vel, d.acc.  A joined
 // pass gathers v and a of a partner in contact (w and al), these forces the stored
-// v* (w*), and the gathers
-// bound a dense bed.  1M packed spheres in no order with 0.9, 1.5, 2.2 and 3.7
-// contacts each, us a step: joined 77, 86, 92 and 100, apart 78, 79, 76 and 78 (with
-// friction, 0.8, 1.2, 2.0 and 4.1 contacts: 163, 194, 240, 291 and 181, 194, 195, 210;
-// in the order of their places: 61, 67, 70, 72 and 75, 76, 74, 74).
+// v* (w*), and where many partners lie far away those gathers bound a dense bed.
+// 1M packed spheres in no order with 0.9, 1.5, 2.2 and 3.7 contacts each, us a step:
+// joined 77, 86, 93 and 100, apart 78, 79, 77 and 78 (with friction, 0.8, 1.2, 2.0 and
+// 4.1 contacts: 163, 194, 227, 283 and 181, 194, 194, 208).  In the order of their
+// places: 61, 67, 71, 74 and 75, 76, 74, 74 (with friction 118, 136, 152, 166 and 159,
+// 166, 165, 169; with 5.9, 171 and 165); 3,000 in no order with 1.6 contacts 13.0 and
+// 13.4.
 template <bool kFric, bool kPartial>
 __global__ void __launch_bounds__(kStepMaxThreads, 1)
 k_advance_apart(const __grid_constant__ DevState s, const __grid_constant__ DemDev d,
@@ -703,9 +705,13 @@ k_advance_apart(const __grid_constant__ DevState s, const __grid_constant__ DemD
     flush_work(s);
 }
 
-// The contacts of a sample of the particles, 32 to a warp from places spread over the
-// arrays, for the choice between the two: contacts in the upper half of *out
-// (host memory), particles in the lower.  One block.
+// How much the contacts of a sample of the particles, 32 to a warp from places spread
+// over the arrays, speak for the second form: a contact with a partner more than
+// kFar places away (whose sector no other particle of the block has asked for) two, with
+// friction any other contact one.  The sum in the upper half of *out (host
+// memory), the particles in the lower.  One block.
+constexpr int kFar = 16384;   // 256 KB of positions, an L1
+
 __global__ void __launch_bounds__(1024)
 k_sample(DemDev d, unsigned long long *out)
 {
@@ -723,7 +729,8 @@ k_sample(DemDev d, unsigned long long *out)
         unsigned long long n = 0;
         for (int e = 0; e < len; ++e) {
             const int j = d.rows.col[off + e];
-            n += j >= 0 && may_touch(xi, d.pos[j]);
+            if (j >= 0 && may_touch(xi, d.pos[j]))
+                n += abs(i - j) > kFar ? 2 : d.omega ? 1 : 0;
         }
         atomicAdd(&sum, (n << 32) + 1);
     }
@@ -900,7 +907,7 @@ auto advance_kernel(const dem_ctx *c, bool apart)
     return c->d.omega ? k_advance<true, false> : k_advance<false, false>;
 }
 
-// Asks for the contacts of a sample of the particles.  The answer is there when
+// Asks for a sample of the contacts.  The answer is there when
 // the stream has come to it; until then the last one stands (both forms of the
 // steps give the same results).
 cudaError_t ask_sample(dem_ctx *c)
@@ -913,13 +920,14 @@ cudaError_t ask_sample(dem_ctx *c)
 
 constexpr int64_t kSampleEvery = 500;   // steps (the sample takes as long as one or two)
 
-// Whether the particles have many contacts: one and a half each, in the sample.
+// Whether the particles have many contacts: one and a half far ones each, in the
+// sample, or with friction three of any kind.
 bool many_contacts(const dem_ctx *c)
 {
     if (!c->sample) return false;
     const unsigned long long v = *(volatile unsigned long long *)c->sample;
-    const unsigned contacts = (unsigned)(v >> 32), seen = (unsigned)v;
-    return seen > 0 && 2 * contacts >= 3 * seen;
+    const unsigned sum = (unsigned)(v >> 32), seen = (unsigned)v;
+    return seen > 0 && sum >= 3 * seen;
 }
 
 // Whether the steps keep their forces apart.  (Mirrored velocities cannot be worked

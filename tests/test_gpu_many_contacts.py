@@ -1,6 +1,8 @@
 """dem_advance where the particles have many contacts: its steps then keep the
-forces apart from the half-steps (a launch chooses by a sample of the contacts,
-taken at the start, after dem_set_state and every 500 steps).
+forces apart from the half-steps.  With specular walls they always do; else a launch
+chooses by a sample of the contacts, taken at the start, after dem_set_state and
+every 500 steps: one and a half with partners that lie far away in the arrays, or
+with friction three of any kind.
 
 Both forms and the phases use the same roundings, and only the order of a row's
 entries, which two contexts need not share, orders a force sum.  So the results are
@@ -25,12 +27,12 @@ def _lvb():
     return lvb
 
 
-def squares(n, mu=0.0, wall="box", seed=3, apart=0.0):
+def squares(n, mu=0.0, wall="box", seed=3, apart=0.0, shuffled=False):
     """Squares A B C D of spheres of 1 mm, 8 mm apart: A and B (along x) overlap by
     2 um, D above A, C above B and C beside D are 0.04 um from touching.  D and C
     move up, away from each other, A and B down, so those distances only grow, and in
     101 steps of 1 us at up to 8 m/s nobody comes near another square.
-    apart: by how much more B and C stand off along x."""
+    apart: by how much more B and C stand off along x.  shuffled: in no order."""
     rng = np.random.default_rng(seed + n)
     k, w = np.arange(n) // 4, np.arange(n) % 4
     side = int(np.ceil((k[-1] + 1) ** (1 / 3)))
@@ -47,6 +49,9 @@ def squares(n, mu=0.0, wall="box", seed=3, apart=0.0):
     vel[:, 1] = np.where(w >= 2, vy, -0.3 * vy)
     vel[:, 2] = rng.uniform(-4.0, 4.0, size=n)
     s = scenes.packed(n=1)
+    if shuffled:
+        order = rng.permutation(n)
+        pos, vel = pos[order], vel[order]
     s.pos, s.vel, s.mu, s.wall = pos, vel, mu, wall
     s.lo, s.hi = (0.0, 0.0, 0.0), (0.008 * side + 0.002,) * 3
     return s
@@ -80,11 +85,13 @@ def run(dems, calls):
 
 
 @pytest.mark.parametrize("mu", [0.0, 0.5])
-@pytest.mark.parametrize("n", [24, 2048, 2049, 20_000, 160_000])
+@pytest.mark.parametrize("n,wall", [(24, "specular"), (2048, "specular"), (2049, "specular"),
+                                    (20_000, "specular"), (160_000, "box"), (160_000, "specular")])
 @pytest.mark.parametrize("calls", [(1, 1, 2), (40,), (3, 37, 61)])
-def test_squares_are_bitwise_the_phases(n, mu, calls):
+def test_squares_are_bitwise_the_phases(n, wall, mu, calls):
+    # (160,000 in no order: the sample has 1.6 far contacts each)
     lvb = _lvb()
-    a, b = [lvb.DEM(squares(n, mu)) for _ in range(2)]
+    a, b = [lvb.DEM(squares(n, mu, wall=wall, shuffled=True)) for _ in range(2)]
     assert len(a.contact_forces()[0]) == n // 4
     run((a, b), calls)
     equal(lvb, a, b)
@@ -99,7 +106,7 @@ def test_squares_are_bitwise_the_phases(n, mu, calls):
 @pytest.mark.parametrize("threads", [1024, 256])
 def test_triggers_and_rules(trigger, kind, early, threads):
     lvb = _lvb()
-    dems = [lvb.DEM(squares(9000), trigger=trigger, skin_kind=kind,
+    dems = [lvb.DEM(squares(9000, wall="specular"), trigger=trigger, skin_kind=kind,
                     skin_value=0.1 if kind == 1 else 15.0) for _ in range(2)]
     for dem in dems:
         dem.lvb.set_option(lvb.LVB_OPT_BLOCK_THREADS, threads)
@@ -115,7 +122,8 @@ def test_triggers_and_rules(trigger, kind, early, threads):
 @pytest.mark.parametrize("mu", [0.0, 0.5])
 def test_batch_of_squares(mu):
     lvb = _lvb()
-    dems = [lvb.DEM([squares(n, mu, seed=q) for q, n in enumerate((700, 3001, 24, 1900))])
+    sizes = (700, 3001, 24, 1900)
+    dems = [lvb.DEM([squares(n, mu, "specular", seed=q) for q, n in enumerate(sizes)])
             for _ in range(2)]
     a, b = run(dems, (1, 20, 70))
     equal(lvb, a, b)
@@ -169,7 +177,7 @@ def test_state_set_later_is_sampled():
     lvb = _lvb()
     out = []
     for joined in (True, False):
-        s, together = squares(6000, apart=3e-4), squares(6000)
+        s, together = (squares(160_000, apart=d, shuffled=True) for d in (3e-4, 0.0))
         dem = lvb.DEM(s)
         assert len(dem.contact_forces()[0]) == 0
         steps = dem.advance if joined else (lambda m: [dem.step() for _ in range(m)])
