@@ -723,12 +723,12 @@ __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int 
     // the first records of the flagged list.  Many scenes: the scene's own
     // segment of the flagged particles (scenes share one coordinate frame,
     // so the global list would also hold far-away twins)
-    const int seg = s.sc_cnt ? g.first : 0;
     float4 rf0 = make_float4(0.f, 0.f, 0.f, 0.f);
     int jf0 = -1;
     if (e0 < m_dir) {
-        rf0 = (s.sc_cnt ? s.sfref : s.fref)[seg + e0];
-        jf0 = (s.sc_cnt ? s.sfid : s.fid)[seg + e0];
+        const bool own = s.sc_cnt != nullptr;
+        rf0 = own ? s.sfref[g.first + e0] : s.fref[e0];
+        jf0 = own ? s.sfid[g.first + e0] : s.fid[e0];
     }
     if (tw == 0 && lane == 0 && m_dir) atomicAdd(&s_work[1], (unsigned long long)m_dir);
     // whether old entry j leaves row i, and (jr, at sp) whether i leaves row j:
@@ -796,9 +796,12 @@ __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int 
             }
         }
     };
-    // the flagged partners of the direct test (all of this scene)
+    // the flagged partners of the direct test (all of this scene).  (The order of
+    // the tests is the faster one of each form: 2,000 flagged of 200k, 54 against 59
+    // us a step; with history 70 against 64.)
     auto flagged = [&](int j, float4 r) {
-        bool take = pair_hit(qn, r) && j >= 0 && j != i;
+        bool take = kHist ? j >= 0 && j != i && pair_hit(qn, r)
+                          : pair_hit(qn, r) && j >= 0 && j != i;
         if (kHist) take = take && !pair_hit(s.oref[k], s.pold[j]);
         append(take, j);
     };
@@ -859,6 +862,7 @@ __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int 
     while (n_noted > 0);
     // the rest of the flagged list, kDirectUnroll records per lane in flight
     // and nothing else to load
+    const int seg = s.sc_cnt && m_dir > per ? g.first : 0;
     const float4 *lst = (s.sc_cnt ? s.sfref : s.fref) + seg;
     const int *ids = (s.sc_cnt ? s.sfid : s.fid) + seg;
     for (int b0 = per + tw * 32 * kDirectUnroll; b0 < m_dir; b0 += per * kDirectUnroll) {
