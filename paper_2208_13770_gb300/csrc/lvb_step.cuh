@@ -796,12 +796,9 @@ __device__ __forceinline__ void patch_row(const DevState &s, const Team tm, int 
             }
         }
     };
-    // the flagged partners of the direct test (all of this scene).  (The order of
-    // the tests is the faster one of each form: 2,000 flagged of 200k, 54 against 59
-    // us a step; with history 70 against 64.)
+    // the flagged partners of the direct test (all of this scene)
     auto flagged = [&](int j, float4 r) {
-        bool take = kHist ? j >= 0 && j != i && pair_hit(qn, r)
-                          : pair_hit(qn, r) && j >= 0 && j != i;
+        bool take = pair_hit(qn, r) && j >= 0 && j != i;
         if (kHist) take = take && !pair_hit(s.oref[k], s.pold[j]);
         append(take, j);
     };
