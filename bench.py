@@ -259,7 +259,7 @@ def _narrow_phase(n, entries, ms, hbm_peak):
 # headline window, from one ncu capture of the current kernel (mean of the
 # captured launches; the command and the counters are in profiles/).  None
 # when the kernel has changed since the capture.
-NCU_TRAFFIC_BATCHED = 203.61e6   # profiles/k_step_batched512_ncu.txt
+NCU_TRAFFIC_BATCHED = 203.55e6   # profiles/k_step_batched512_ncu.txt
 
 
 # ----------------------------------------------------------------- headline
@@ -771,7 +771,7 @@ def _clumps(lvb, torch, n=400_000, seed=2208_13770 + 21):
     bounding spheres on a jittered lattice at 1.6 median bounding radii (so
     neighbours' bounds overlap); the narrow phase's time per call between
     CUDA events, outputs in device memory (the call includes its input
-    checks and two synchronisations)."""
+    checks and one wait)."""
     rng = np.random.default_rng(seed)
     k = rng.integers(1, 5, size=n)
     off = np.concatenate([[0], np.cumsum(k)]).astype(np.int32)
